@@ -193,6 +193,20 @@ bool env_fused() {
   return e && e[0] == '1';
 }
 
+// Whether the page pass of a launch scores only the pages whose bound can
+// raise R (exact; see bound_kernel).  It needs
+// R alone as output: the maxima per head take every page of every head.
+bool prune_pages(int n, const commitkv_traj *tr, int slices, int g, float *const *headR) {
+  int64_t work = 0;
+  for (int t = 0; t < n; ++t) {
+    if (headR[t]) return false;
+    if (tr[t].S == 0 || tr[t].W == 0 || tr[t].P == 0) continue;
+    if ((int64_t)tr[t].P * tc::kMinPageTokens > tr[t].S) return false;
+    work += (int64_t)slices * cdiv(g * tr[t].W, tc::kRowsPerTile) * tr[t].S;
+  }
+  return work >= tc::kMinPruneWork;
+}
+
 // Flash-pass partial slots the tensor-core path may need for these caches or
 // smaller ones: one per item of the two-launch chunking, or the fused
 // launch's ring (at most kMaxFusedCtas x kPartialRing slots, and at most one
@@ -215,6 +229,8 @@ size_t tc_score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *
     TcCounts c = tc_counts(s, tr[t], tc_chunk_len(1, &tr[t]));
     slots += align_up((size_t)(tr[t].P + 1) * 4) + align_up((size_t)c.nbitem * 32) + kAlign +
              align_up(((size_t)cdiv(tr[t].S, 16) + tr[t].P) * 16);
+    slots += tc::prune_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt) +
+             align_up(tc::prune_item_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt)) + kAlign;
     slices += (size_t)s->layers * s->kv_heads;
   }
   return align_up(tc_partial_slots(s, n_traj, tr) * tc::kPartsPerItem * tc::kRowsPerTile * 132 * 4) +
@@ -426,6 +442,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   for (int b0 = 0; b0 < n_traj; b0 += tc::kMaxTc) {
     int nb = n_traj - b0 < tc::kMaxTc ? n_traj - b0 : tc::kMaxTc;
     memset(&T, 0, sizeof T);
+    T.prune = !fused && !from_stats && prune_pages(nb, trajs + b0, nl * shape->kv_heads, L.batch.g, L.headR + b0);
     T.n_traj = nb;
     T.M = shape->layers;
     T.H = shape->kv_heads;
@@ -458,6 +475,14 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       slot_base += kAlign;
       tt.slot_tab = reinterpret_cast<int4 *>(slot_base);
       slot_base += align_up(((size_t)cdiv(x.S, 16) + x.P) * 16);
+      {
+        const int slices = shape->layers * shape->kv_heads;
+        if (T.prune) {
+          if (!T.n_list_items) T.n_list_items = reinterpret_cast<int *>(slot_base);
+          tc::prune_layout(tt.pr, slot_base + kAlign, x.S, x.P, slices, c.nrt);
+        }
+        slot_base += kAlign + tc::prune_bytes(x.S, x.P, slices, c.nrt);
+      }
       tt.stats = L.stats[t];
       tt.nvis_w = L.nvis_w[t];
       tt.R = L.R[t];
@@ -475,9 +500,15 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       T.item_off_b[i + 1] = T.item_off_b[i] + ib;
       T.row_off[i + 1] = T.row_off[i] + (active ? nl * shape->kv_heads * L.batch.g * x.W : 0);
       T.slice_off[i + 1] = T.slice_off[i] + (active ? nl * shape->kv_heads : 0);
+      T.unit_off[i + 1] = T.unit_off[i] + (active && x.P > 0 ? nl * shape->kv_heads * c.nrt : 0);
       if (active && !tc::build_maps(T.maps[i], L.batch.t[t], shape->layers, shape->kv_heads, shape->q_heads))
         return COMMITKV_ERR_CUDA;
     }
+    // one array of work items for the launch, after its trajectories' regions
+    T.list_items = reinterpret_cast<int4 *>(slot_base);
+    for (int i = 0; i < nb; ++i)
+      slot_base += align_up(tc::prune_item_bytes(trajs[b0 + i].S, trajs[b0 + i].P, shape->layers * shape->kv_heads,
+                                                 T.t[i].nrt));
     e = tc::launch_score_tc(T, hdr, stream, sms);
     if (e != cudaSuccess) return cuda_status(e);
   }

@@ -8,7 +8,16 @@
 //            chunk's (max, sum, count, O) per probe row.
 //   combine  merges a slice's chunk partials into the row stats
 //            (m, l, n, o) of the whole cache.
-//   slots    per trajectory, the prefix count of 16-token slots per page.
+//   prep     per trajectory, the prefix count of 16-token slots per page.
+//   bounds   an upper bound of every page's effect on the 128 probe rows of
+//            a unit, from the row sums over pages that pass A left (large
+//            calls without maxima per head): pass B then scores only the
+//            pages of a unit that can raise R, first those of the unit with
+//            the largest bound, then those whose bound is above the effects
+//            found.  On 36 layers of 16K + 2K tokens (pages of 32): page pass
+//            1,495 us, instead bounds 61, lists 18, page pass over the rest
+//            250, and pass A 884 -> 1,099 us for the sums; 32K + 4K: scoring
+//            4.26 -> 2.6 ms.
 //   pass B   persistent, over tiles of 8 slots: every page is loaded as
 //            16-row TMA boxes into slots of its own, so one page's columns
 //            never share a 16-wide MMA k-block with another page.
@@ -41,6 +50,7 @@ constexpr int NVB = 2;   // pass B: V stages
 constexpr int SLOT = 16;
 constexpr int SLOTS = BT / SLOT;  // slots per pass-B tile
 constexpr int NFIFO = 16;         // page-sum FIFO depth (>= 2 x SLOTS)
+constexpr int kListSlotsPerItem = 64;  // slots per work item of the pruned page pass
 constexpr uint64_t kWait = 1000000000ull;
 constexpr float kLazy = 8.0f;     // rescale O when the max grows by > 2^8
 constexpr int kRing = kPartialRing;  // partial slots per flash CTA of the fused launch
@@ -151,6 +161,27 @@ __device__ __forceinline__ void signal_add(uint32_t *p, int lane) {
 template <bool FUSED>
 __device__ __forceinline__ void merge_row(const TcLaunch &L, int t, int li, int kvh, int row, int lane);
 
+// Upper bound of |v| of row `tok` of a V tile in shared memory.
+__device__ __forceinline__ __half norm_bound(const uint8_t *tile, int tok) {
+  __nv_bfloat162 acc[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc[k] = __floats2bfloat162_rn(0.0f, 0.0f);
+#pragma unroll
+  for (int c = 0; c < D / 8; ++c) {
+    const uint4 w = *reinterpret_cast<const uint4 *>(tile + (c >> 3) * kHalf + sw128_offset(tok, c & 7));
+    const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const __nv_bfloat162 v2 = *reinterpret_cast<const __nv_bfloat162 *>(&x[k]);
+      acc[k] = __hfma2(v2, v2, acc[k]);
+    }
+  }
+  float n2 = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) n2 += __low2float(acc[k]) + __high2float(acc[k]);
+  return __float2half_ru(sqrtf(n2 * 1.07f) + 2e-18f);
+}
+
 // ============================================================== pass A
 // Two softmax warpgroups take alternate tiles of a chunk (global tile g goes
 // to warpgroup g & 1), each with its own S/P buffer, running max, sum and
@@ -164,6 +195,8 @@ struct SmemA {
   alignas(1024) uint8_t k[NKB][kTileBytes];
   alignas(1024) uint8_t v[NVB][kTileBytes];
   int pos[2][4][BT];  // per softmax warp: positions of the current tile
+  float4 gs[2][4][BM];  // SUMS: per S/P buffer, 32-column chunk and row, the sums of the chunk's groups of eight columns
+  float mused[2][BM];   // SUMS: per S/P buffer and row, the reference max of P
   float4 pub[BM];     // fused launch: warpgroup 1's (reference max, sum, count, true max) of the item, per row
   uint64_t q_full, q_empty, k_full[NKB], k_empty[NKB], v_full[NVB], v_empty[NVB], s_full[2], s_empty[2], p_full[2],
       pv_done[2], o_full[2], o_empty[2], drain, drain2, pub_full, pub_empty;
@@ -212,7 +245,17 @@ __device__ __forceinline__ void issue_pv_step(uint32_t tm, uint32_t d_col, const
   mma_bf16_ts(tm + d_col, tm + p_col(b, ks, 1), bd, idesc, 1u);
 }
 
-template <bool FUSED>
+// log2 on the special-function unit (log2 0 = -inf).
+__device__ __forceinline__ float fast_log2(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// SUMS: also what the pruned page pass needs: log2 of every row's exp-sum
+// over every page (one piece per tile that the page touches) and an upper
+// bound of every token's |v|.
+template <bool FUSED, bool SUMS>
 __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uint8_t *smem_raw, const int cta,
                                            const int ncta) {
   SmemA &sm = *reinterpret_cast<SmemA *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -230,11 +273,11 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
     }
     for (int s = 0; s < NVB; ++s) {
       mbar_init(&sm.v_full[s], 1);
-      mbar_init(&sm.v_empty[s], 1);
+      mbar_init(&sm.v_empty[s], SUMS ? 5 : 1);  // P V and, with SUMS, the four warps of the page sums
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sm.s_full[b], 1);
-      mbar_init(&sm.s_empty[b], 1);
+      mbar_init(&sm.s_empty[b], SUMS ? 5 : 1);
       mbar_init(&sm.p_full[b], 4);
       mbar_init(&sm.pv_done[b], 1);
       mbar_init(&sm.o_full[b], 1);
@@ -256,12 +299,13 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
   const uint32_t tm = sm.tmem;
 
   // warpgroup 0: TMA producer, P V issuer, Q K^T issuer, one idle warp; 1 and
-  // 2: softmax of the even and the odd tiles.  Register budget per thread:
-  // 104 + 2 x 200 = the launch's 3 x 168 (the issuers' loops spill below 104;
-  // the softmax needs no more than 200).
+  // 2: softmax of the even and the odd tiles; 3 (SUMS): page sums and token norms.  Register
+  // budget per thread: 104 + 2 x 200 = the launch's 3 x 168, with SUMS
+  // 72 + 2 x 176 + 88 = 4 x 128.
   if (warp < 4) {
     if (FUSED) regs_dec<48>();
-    else regs_dec<104>();  // warp 3 stays idle
+    else if (SUMS) regs_dec<72>();
+    else regs_dec<104>();
     if (warp == 0) {
       // ------------------------------------------------------------ TMA producer
       if (lane == 0) {
@@ -398,6 +442,7 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
   } else if (warp < 12) {
     // ------------------------------------------------------------ softmax (warps 4..11)
     if (FUSED) regs_inc<208>();
+    else if (SUMS) regs_inc<176>();
     else regs_inc<200>();
     const int hb = (warp - 4) >> 2;   // this warpgroup's tiles: g & 1 == hb
     const int wq = warp & 3;          // TMEM lane quarter of this warp
@@ -499,9 +544,7 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
         const float neg_m = m_used == -INFINITY ? 0.0f : -m_used;
         // sweep 2: p = 2^(s c - m) on the visible columns (2^-inf = 0), the row
         // sum, and P as the (hi, lo) bf16 pair over the S columns just read
-        float pacc[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) pacc[k] = 0.0f;
+        float ps = 0.0f;
 #pragma unroll 1
         for (int c0 = 0; c0 < BT; c0 += 32) {
           float x[32];
@@ -516,15 +559,18 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           }
 #pragma unroll
           for (int i = 0; i < 32; ++i) x[i] = fast_exp2(fmaf(x[i], L.scale_log2, neg_m));
+          float gs[4];  // sums of the four groups of eight columns
 #pragma unroll
-          for (int i = 0; i < 32; i += 8)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) pacc[k] += x[i + k];
+          for (int q = 0; q < 4; ++q)
+            gs[q] = ((x[8 * q] + x[8 * q + 1]) + (x[8 * q + 2] + x[8 * q + 3])) +
+                    ((x[8 * q + 4] + x[8 * q + 5]) + (x[8 * q + 6] + x[8 * q + 7]));
+          ps += (gs[0] + gs[1]) + (gs[2] + gs[3]);
+          if constexpr (SUMS) sm.gs[b][c0 / 32][row] = make_float4(gs[0], gs[1], gs[2], gs[3]);
           uint32_t pk[32];
           split_pack32(x, pk);
           tmem_st32(tm + lane_base + b * BT + c0, pk);
         }
-        float ps = ((pacc[0] + pacc[1]) + (pacc[2] + pacc[3])) + ((pacc[4] + pacc[5]) + (pacc[6] + pacc[7]));
+        if constexpr (SUMS) sm.mused[b][row] = m_used;
         tmem_wait_st();
         lsum += ps;
         tc_fence_before();
@@ -616,6 +662,98 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
         it += ntile;
       }
     }
+  } else if (SUMS) {
+    // ------------------------------------------------------------ page sums, norms (warps 12..15)
+    // Per tile, one thread per token: the bound of |v|; then, one thread per
+    // probe row (TMEM lane) as in the softmax: walks the sums of eight
+    // columns that the softmax left in shared memory, cuts them at the page
+    // starts and ends (a cut inside a group reads the group's P from tensor
+    // memory) and writes log2 of the row's sum over every piece of a page.
+    // Here, not in the softmax: there the same work lay on every tile's
+    // chain (flash pass 39.8 -> 57.3 ms on 64 layers of 128K tokens and 512
+    // probe rows).
+    regs_dec<88>();
+    const int wq = warp & 3, row = wq * 32 + lane;
+    const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int item = cta; item < n_items && ok; item += ncta) {
+      const ItemA a = decode_a(L, item);
+      const TcTraj &tr = L.t[a.t];
+      const int t0 = a.c * L.chunk_len, t1 = min(tr.S, t0 + L.chunk_len);
+      const int ntile = (t1 - t0 + BT - 1) / BT;
+      __half *norms = tr.pr.vnorm + (int64_t)(a.li * L.H + a.kvh) * ((tr.S + BT - 1) / BT * BT) + t0 + row;
+      __half *piece_row =
+          tr.pr.pieces + (int64_t)((a.li * L.H + a.kvh) * tr.nrt + a.rt) * tr.pr.npiece * BM + row;
+      const int2 *tiles = tr.pr.tile + t0 / BT;
+      const uint2 *cuts = tr.pr.cuts + t0 / 32;
+#pragma unroll 1
+      for (int j = 0; j < ntile; ++j) {
+        const uint32_t g = it + j;
+        const int s2 = g % NVB, b = g & 1;
+        const int2 tile = __ldg(&tiles[j]);
+        const uint2 cut4 = __ldg(&cuts[4 * j + (lane & 3)]);  // lane i: chunk i mod 4
+        if (!__all_sync(0xffffffffu, mbar_wait(&sm.v_full[s2], (g / NVB) & 1, kWait, abort_flag))) {
+          ok = false;
+          break;
+        }
+        if (a.rt == 0) norms[j * BT] = norm_bound(sm.v[s2], row);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.v_empty[s2]);
+        if (!__all_sync(0xffffffffu, mbar_wait(&sm.p_full[b], (g >> 1) & 1, kWait, abort_flag))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        __half *dst = piece_row + (int64_t)tile.x * BM;
+        const float mu = sm.mused[b][row];
+        // run: the row's sum before the chunk; base: before the segment being
+        // walked; part: the part of base that comes from a cut group.  A sum
+        // of P is within 2^-16 of its terms' sum, a difference of two running
+        // sums within 2^-21 of the larger: added on top.
+        float run = 0.0f, base = 0.0f, part = 0.0f;
+        auto put = [&](float end, float end_part) {
+          const float s = fmaxf(end - base, 0.0f) + fmaf(end, 5e-7f, (end_part + part) * 2e-5f);
+          *dst = __float2half_ru(fast_log2(s) + mu);
+          dst += BM;
+        };
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+          const float4 gs = sm.gs[b][c][row];
+          uint32_t m = __shfl_sync(0xffffffffu, cut4.x, c);
+          const uint32_t ends = __shfl_sync(0xffffffffu, cut4.y, c);
+#pragma unroll 1
+          while (m) {
+            const int at = __ffs(m) - 1, q = at >> 3, k = at & 7;
+            m &= m - 1;
+            float p = 0.0f;
+            if (k) {
+              uint32_t hi[4], lo[4];
+              tmem_ld4(tm + lane_base + b * BT + 32 * c + 4 * q, hi);
+              tmem_ld4(tm + lane_base + b * BT + 32 * c + 16 + 4 * q, lo);
+              tmem_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 7; ++e) {
+                const uint32_t h = hi[e >> 1], w = lo[e >> 1];
+                const float x = e & 1 ? __uint_as_float(h & 0xffff0000u) + __uint_as_float(w & 0xffff0000u)
+                                      : __uint_as_float(h << 16) + __uint_as_float(w << 16);
+                p += e < k ? x : 0.0f;
+              }
+            }
+            const float end = run + (q > 0 ? gs.x : 0.0f) + (q > 1 ? gs.y : 0.0f) + (q > 2 ? gs.z : 0.0f) + p;
+            if ((ends >> at) & 1u) put(end, p);
+            base = end;
+            part = p;
+          }
+          run += (gs.x + gs.y) + (gs.z + gs.w);
+        }
+        if (tile.y) put(run, 0.0f);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.s_empty[b]);
+      }
+      it += ntile;
+    }
   } else if (FUSED) {
     // ------------------------------------------------------------ merge (warps 12..15, fused launch only)
     // For each item of this CTA, once every item of its slice has written
@@ -644,9 +782,10 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
   }
 }
 
-__global__ void __launch_bounds__(384, 1) pass_a_tc(const __grid_constant__ TcLaunch L, WsHeader *hdr) {
+template <bool SUMS>
+__global__ void __launch_bounds__(SUMS ? 512 : 384, 1) pass_a_tc(const __grid_constant__ TcLaunch L, WsHeader *hdr) {
   extern __shared__ uint8_t smem_raw[];
-  flash_body<false>(L, hdr, smem_raw, blockIdx.x, gridDim.x);
+  flash_body<false, SUMS>(L, hdr, smem_raw, blockIdx.x, gridDim.x);
 }
 
 
@@ -709,7 +848,14 @@ __device__ __forceinline__ void merge_row(const TcLaunch &L, int t, int li, int 
   float *dst = tr.stats + (((int64_t)l * L.Hq + h) * tr.W + w) * (D + 4);
   if (lane == 0)
     *reinterpret_cast<float4 *>(dst) = make_float4(m == -INFINITY ? m : m * 0.69314718055994531f, lsum, n, 0.0f);
-  *reinterpret_cast<float4 *>(dst + 4 + lane * 4) = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
+  const float4 on = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
+  *reinterpret_cast<float4 *>(dst + 4 + lane * 4) = on;
+  if (!FUSED && L.prune) {  // the terms of bound_kernel; the max as the page pass reads it back
+    const float n2 = warp_sum(fmaf(on.x, on.x, fmaf(on.y, on.y, fmaf(on.z, on.z, on.w * on.w))));
+    if (lane == 0)
+      tr.pr.aux[((int64_t)(li * L.H + kvh) * tr.nrt + rt) * BM + rl] =
+          make_float4(m == -INFINITY ? m : (m * 0.69314718055994531f) * 1.4426950408889634f, lsum, sqrtf(n2), 0.0f);
+  }
 }
 
 // One warp per probe row of the selected layers (the two-launch path).
@@ -728,65 +874,111 @@ __global__ void __launch_bounds__(256) combine_tc(const __grid_constant__ TcLaun
 // ============================================================== prep
 // Per trajectory, once per call:
 //   slot_off[E] = sum over F < E of ceil(len_F / 16), slot_off[P] = total
-//   (a page that fails the table checks gets no slot and an error is recorded);
-//   slot_tab[slot] = {first token, valid tokens, page, first/last flags and
-//   the page's rank among the pages with slots} for every 16-token slot;
+//   (a page that fails the table checks gets no slot and an error is recorded;
+//   the pages with slots are disjoint, which bounds the tables);
+//   slot_tab[slot] = {first token, valid tokens, page, first/last flags} for
+//   every 16-token slot;
 //   the pass-B work items: item k takes the pages whose first slot lies in
 //   [k * slots_per_item, (k + 1) * slots_per_item);
 //   vis_all = number of leading resident tokens visible to every probe row
 //   (positions increase, so this is a prefix); nvis_w[w] = number of resident
 //   tokens visible to window position w.
+// For a pruned launch also where the flash pass cuts its row sums (cuts,
+// tile, piece_off: a page with slots has one piece per 128-token tile that it
+// touches), and the counters of the list passes cleared.
 __global__ void __launch_bounds__(1024) prep_kernel(const __grid_constant__ TcLaunch L, WsHeader *hdr) {
   const TcTraj &tr = L.t[blockIdx.x];
   int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
-  // one scan gives both the slot offsets (low 32 bits) and the rank of each
-  // page among the pages that have slots (high 32 bits)
-  __shared__ unsigned long long s_w64[32];
-  __shared__ unsigned long long s_b64;
-  if (threadIdx.x == 0) s_b64 = 0ull;
+  // one scan gives both the slot offsets (low 32 bits) and the piece offsets
+  // (high 32 bits)
+  __shared__ unsigned long long s_w[32], s_b;
+  __shared__ int s_end[32], s_bend;  // largest end of the pages seen so far
+  if (threadIdx.x == 0) s_b = 0ull, s_bend = 0;
+  const bool prune = L.prune != 0 && tr.S > 0 && tr.W > 0;
+  if (prune) {
+    const int ntile = (tr.S + BT - 1) / BT;
+    for (int i = threadIdx.x; i < 4 * ntile; i += 1024) tr.pr.cuts[i] = make_uint2(0u, 0u);
+    for (int i = threadIdx.x; i < ntile; i += 1024) tr.pr.tile[i] = make_int2(0x7fffffff, 0);
+  }
+  if (L.prune && blockIdx.x == 0 && threadIdx.x < 2) L.n_list_items[threadIdx.x] = 0;
   __syncthreads();
   for (int c0 = 0; c0 < tr.P; c0 += 1024) {
     int E = c0 + threadIdx.x;
-    int ns = 0, ps = 0, pl = 0;
+    int ns = 0, ps = 0, pl = 0, end_incl = 0;
+    bool span = false;
     if (E < tr.P) {
       ps = tr.ps[E];
       pl = tr.pl[E];
-      bool bad = pl < 0 || ps < 0 || ps > tr.S - pl || (E > 0 && ps < tr.ps[E - 1] + tr.pl[E - 1]);
+      span = pl >= 0 && ps >= 0 && ps <= tr.S - pl;
+      end_incl = span ? ps + pl : 0;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, end_incl, o);
+      if (lane >= o) end_incl = max(end_incl, y);
+    }
+    if (lane == 31) s_end[wid] = end_incl;
+    __syncthreads();
+    int end_before = __shfl_up_sync(0xffffffffu, end_incl, 1);
+    if (lane == 0) end_before = 0;
+    for (int w = 0; w < wid; ++w) end_before = max(end_before, s_end[w]);
+    end_before = max(end_before, s_bend);
+    if (E < tr.P) {
+      const bool bad = !span || ps < end_before;
       if (bad) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, E);
       ns = bad ? 0 : (pl + SLOT - 1) / SLOT;
     }
-    const unsigned long long v = ((unsigned long long)(ns > 0) << 32) | (unsigned)ns;
+    const int np = ns > 0 ? (ps + pl - 1) / BT - ps / BT + 1 : 0;
+    const unsigned long long v = ((unsigned long long)np << 32) | (unsigned)ns;
     unsigned long long x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
     }
-    if (lane == 31) s_w64[wid] = x;
+    if (lane == 31) s_w[wid] = x;
     __syncthreads();
     if (wid == 0) {
-      unsigned long long w = s_w64[lane];
+      unsigned long long w = s_w[lane];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
         if (lane >= o) w += y;
       }
-      s_w64[lane] = w;
+      s_w[lane] = w;
     }
     __syncthreads();
-    const unsigned long long excl = s_b64 + (wid ? s_w64[wid - 1] : 0ull) + x - v;
+    const unsigned long long excl = s_b + (wid ? s_w[wid - 1] : 0ull) + x - v;
     if (E < tr.P) {
-      const int off = (int)(excl & 0xffffffffull), rank = (int)(excl >> 32);
+      const int off = (int)(excl & 0xffffffffull), piece = (int)(excl >> 32);
       tr.slot_off[E] = off;
       for (int sub = 0; sub < ns; ++sub)
         tr.slot_tab[off + sub] = make_int4(ps + sub * SLOT, min(SLOT, pl - sub * SLOT), E,
-                                           (sub == 0 ? 1 : 0) | (sub + 1 == ns ? 2 : 0) | (rank << 2));
+                                           (sub == 0 ? 1 : 0) | (sub + 1 == ns ? 2 : 0));
+      if (prune) tr.pr.piece_off[E] = piece;
+      if (prune && np > 0) {
+        const int end = ps + pl;
+        atomicOr(&tr.pr.cuts[ps / 32].x, 1u << (ps % 32));
+        if (end % BT) {
+          atomicOr(&tr.pr.cuts[end / 32].x, 1u << (end % 32));
+          atomicOr(&tr.pr.cuts[end / 32].y, 1u << (end % 32));
+        }
+        for (int k = 0; k < np; ++k) {
+          atomicMin(&tr.pr.tile[ps / BT + k].x, piece + k);
+          if (k + 1 < np || end % BT == 0) tr.pr.tile[ps / BT + k].y = 1;
+        }
+      }
     }
     __syncthreads();
-    if (threadIdx.x == 0) s_b64 += s_w64[31];
+    if (threadIdx.x == 1023) s_b += s_w[31], s_bend = max(end_before, end_incl);
     __syncthreads();
   }
-  if (threadIdx.x == 0) tr.slot_off[tr.P] = (int)(s_b64 & 0xffffffffull);
+  if (threadIdx.x == 0) {
+    const int nslot = (int)(s_b & 0xffffffffull);
+    tr.slot_off[tr.P] = nslot;
+    tr.prep->nitem = (nslot + L.slots_per_item - 1) / L.slots_per_item;
+    if (prune) tr.pr.piece_off[tr.P] = (int)(s_b >> 32);
+  }
   __syncthreads();
   for (int k = threadIdx.x; k < tr.nbitem; k += 1024) {
     int lo = k * L.slots_per_item, hi = lo + L.slots_per_item;
@@ -834,6 +1026,36 @@ __global__ void __launch_bounds__(1024) prep_kernel(const __grid_constant__ TcLa
   }
 }
 
+// Work items of the page pass, from the number of slots that the pages really
+// have.  The host knows an upper bound only; with items counted from it the
+// empty ones fell on some CTAs more than on others (page pass of 36 layers of
+// 26.5K tokens 1,855 us, 990 us with the real counts).
+struct ItemCount {
+  int off[kMaxTc + 1];  // prefix per trajectory
+  int per[kMaxTc];      // items per unit
+};
+// Called by all 32 lanes of one warp.
+__device__ __forceinline__ void count_items(const TcLaunch &L, ItemCount &c) {
+  const int lane = threadIdx.x % 32;
+  int per = 0, n = 0;
+  if (lane < L.n_traj) {
+    const TcTraj &tr = L.t[lane];
+    if (L.item_off_b[lane + 1] > L.item_off_b[lane]) {
+      per = tr.prep->nitem;
+      n = per * L.n_layers * L.H * tr.nrt;
+    }
+    c.per[lane] = per;
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, n, o);
+    if (lane >= o) n += y;
+  }
+  if (lane == 0) c.off[0] = 0;
+  if (lane < L.n_traj) c.off[lane + 1] = n;
+}
+static_assert(kMaxTc <= 32, "one lane per trajectory");
+
 // ============================================================== pass B
 // TMEM columns: S/P buffers at 0 and 128 (as in pass A), page accumulators
 // U[0] at 256 and U[1] at 384.
@@ -856,6 +1078,7 @@ struct SmemB {
   float fifo_s[NFIFO][BM];  // per page: S_E of every row
   int fifo_n[NFIFO][BM];    // per page: visible count of every row
   int fifo_page[NFIFO];
+  ItemCount ic;
   uint64_t q_full, q_empty, k_full[NKB], k_empty[NKB], meta_empty[NKB], v_full[NVB], v_empty[NVB], s_full[2],
       s_empty[2], p_full[2], acc_full[2], acc_empty[2], fifo_full[NFIFO], fifo_empty[NFIFO], drain[2], drain2;
   uint32_t tmem;
@@ -863,37 +1086,56 @@ struct SmemB {
 };
 
 struct ItemB {
-  int t, l, kvh, rt, k, li;
-  int E0, E1;        // pages [E0, E1)
-  int slot0, nslot;  // slots of those pages
+  int t, l, kvh, rt, li;
+  int npages;          // pages of the item (with slots)
+  int nslot;           // slots of those pages
+  const int4 *stab;    // their slot records, or the whole table with
+  const int32_t *ids;  // the records' indices (LIST)
 };
 
-__device__ __forceinline__ ItemB decode_b(const TcLaunch &L, int item) {
+// LIST: the item is a run of a unit's slot list (pass 0 or 1 of the pruned
+// page pass); otherwise a run of consecutive pages.
+template <bool LIST>
+__device__ __forceinline__ ItemB decode_b(const TcLaunch &L, const ItemCount &ic, int item) {
   ItemB b;
-  b.t = traj_of(L.item_off_b, L.n_traj, item);
-  const TcTraj &tr = L.t[b.t];
-  int local = item - L.item_off_b[b.t];
-  b.rt = local % tr.nrt;
-  local /= tr.nrt;
-  b.k = local % tr.nbitem;
-  local /= tr.nbitem;
-  b.kvh = local % L.H;
-  b.li = local / L.H;
+  if constexpr (LIST) {
+    const int4 e = L.list_items[item];
+    b.t = traj_of(L.unit_off, L.n_traj, e.x);
+    const TcTraj &tr = L.t[b.t];
+    int local = e.x - L.unit_off[b.t];
+    b.ids = tr.pr.list + (int64_t)local * tr.pr.cap + e.y;
+    b.stab = tr.slot_tab;
+    b.rt = local % tr.nrt;
+    local /= tr.nrt;
+    b.kvh = local % L.H;
+    b.li = local / L.H;
+    b.nslot = e.z;
+    b.npages = e.w;
+  } else {
+    b.t = traj_of(ic.off, L.n_traj, item);
+    const TcTraj &tr = L.t[b.t];
+    int local = item - ic.off[b.t];
+    b.rt = local % tr.nrt;
+    local /= tr.nrt;
+    const int k = local % ic.per[b.t];
+    local /= ic.per[b.t];
+    b.kvh = local % L.H;
+    b.li = local / L.H;
+    const int4 e = tr.items[2 * k];
+    b.stab = tr.slot_tab + e.z;
+    b.ids = nullptr;
+    b.nslot = e.w;
+    b.npages = tr.items[2 * k + 1].x;
+  }
   b.l = L.layer_ids[b.li];
-  int4 e = tr.items[2 * b.k];
-  b.E0 = e.x;
-  b.E1 = e.y;
-  b.slot0 = e.z;
-  b.nslot = e.w;
   return b;
 }
 
-template <bool FUSED>
+template <bool FUSED, bool LIST>
 __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint8_t *smem_raw, const int cta,
-                                          const int ncta) {
+                                          const int ncta, const int n_list) {
   SmemB &sm = *reinterpret_cast<SmemB *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int n_items = L.item_off_b[L.n_traj];
   volatile int *abort_flag = &sm.abort_flag;
 
   if (threadIdx.x == 0) {
@@ -933,10 +1175,12 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
     tmem_alloc(&sm.tmem, 512);
     tmem_relinquish();
   }
+  if (!LIST && warp == 2) count_items(L, sm.ic);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = sm.tmem;
+  const int n_items = LIST ? n_list : sm.ic.off[L.n_traj];
 
   // warpgroup 0: TMA producer, two P V issuers (warps 1 and 3), Q K^T issuer; 1: softmax;
   // 2 and 3: epilogue.  Each branch first sets its warpgroup's register
@@ -951,16 +1195,14 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
       // issue the copies of the runs of slots that start at them.
       uint64_t pol = policy_evict_first();
       uint32_t it = 0, n_local = 0, n_k = 0, n_v = 0;  // tiles; Q, K and V copies issued
-      int po_base = 0;  // page ordinal of the item's first page
+      int po_next = 0;  // page ordinal of the next page to start
       bool stop = false;
       for (int item = cta; item < n_items && !stop; item += ncta) {
         if (*abort_flag) break;
-        ItemB bi = decode_b(L, item);
+        ItemB bi = decode_b<LIST>(L, sm.ic, item);
         if (bi.nslot == 0) continue;
         const TcTraj &tr = L.t[bi.t];
         const TcMaps &mp = L.maps[bi.t];
-        const int4 *stab = tr.slot_tab + bi.slot0;
-        const int rank0 = stab[0].w >> 2;  // slotted-page rank of the item's first page
         const int vis_all = tr.prep->vis_all;
         if (n_local > 0 && !__all_sync(0xffffffffu, mbar_wait(&sm.q_empty, (n_local - 1) & 1, kWait, abort_flag))) {
           stop = true;
@@ -1009,12 +1251,14 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
           if (!__all_sync(0xffffffffu, w_ok)) return false;
           int sl = j * SLOTS + lane;
           bool valid = lane < SLOTS && sl < bi.nslot;
-          int4 rec = valid ? stab[sl] : make_int4(0, 0, -1, 0);
+          int4 rec = valid ? bi.stab[LIST ? bi.ids[sl] : sl] : make_int4(0, 0, -1, 0);
+          const unsigned starts = __ballot_sync(0xffffffffu, valid && (rec.w & 1));
           SlotMeta mt;
           mt.tok0 = rec.x;
           mt.nv = valid ? rec.y : 0;
-          mt.po = valid ? po_base + (rec.w >> 2) - rank0 : -1;
+          mt.po = valid ? po_next + __popc(starts & ((2u << lane) - 1u)) - 1 : -1;
           mt.flags = valid ? rec.w & 3 : 0;
+          po_next += __popc(starts);
           if (lane < SLOTS) {
             sm.meta[s3][lane] = mt;
             sm.page_of[s3][lane] = rec.z;
@@ -1053,7 +1297,6 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
           else if (!load_v(it + j)) stop = true;
         }
         it += ntile;
-        po_base += tr.items[2 * bi.k + 1].x;
       }
       if (lane == 0 && *abort_flag) {
         // let the copies already issued land before the CTA leaves
@@ -1073,7 +1316,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
         uint32_t it = 0;
         bool ok = true;
         for (int item = cta; item < n_items && ok; item += ncta) {
-          ItemB bi = decode_b(L, item);
+          ItemB bi = decode_b<LIST>(L, sm.ic, item);
           if (bi.nslot == 0) continue;
           int ntile = (bi.nslot + SLOTS - 1) / SLOTS;
           for (int j = 0; j < ntile && ok; ++j) {
@@ -1119,7 +1362,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
         uint32_t it = 0, n_local = 0;
         bool ok = true;
         for (int item = cta; item < n_items && ok; item += ncta) {
-          ItemB bi = decode_b(L, item);
+          ItemB bi = decode_b<LIST>(L, sm.ic, item);
           if (bi.nslot == 0) continue;
           int ntile = (bi.nslot + SLOTS - 1) / SLOTS;
           if (!mbar_wait(&sm.q_full, n_local & 1, kWait, abort_flag)) break;
@@ -1159,7 +1402,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
     int n_cur = 0;
     bool ok = true;
     for (int item = cta; item < n_items && ok; item += ncta) {
-      ItemB bi = decode_b(L, item);
+      ItemB bi = decode_b<LIST>(L, sm.ic, item);
       if (bi.nslot == 0) continue;
       const TcTraj &tr = L.t[bi.t];
       int rows = L.g * tr.W;
@@ -1298,7 +1541,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
     int po = 0;
     bool ok = true;
     for (int item = cta; item < n_items && ok; item += ncta) {
-      ItemB bi = decode_b(L, item);
+      ItemB bi = decode_b<LIST>(L, sm.ic, item);
       if (bi.nslot == 0) continue;
       const TcTraj &tr = L.t[bi.t];
       int rows = L.g * tr.W;
@@ -1331,8 +1574,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
         }
         onorm = sqrtf(ss);
       }
-      int npages = tr.items[2 * bi.k + 1].x;
-      for (int k = 0; k < npages && ok; ++k, ++po) {
+      for (int k = 0; k < bi.npages && ok; ++k, ++po) {
         if ((po & 1) != par) continue;
         int f = po % NFIFO;
         if (!__all_sync(0xffffffffu, mbar_wait(&sm.fifo_full[f], (po / NFIFO) & 1, kWait, abort_flag) &&
@@ -1389,7 +1631,210 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
 
 __global__ void __launch_bounds__(512, 1) pass_b_tc(const __grid_constant__ TcLaunch L, WsHeader *hdr) {
   extern __shared__ uint8_t smem_raw[];
-  page_body<false>(L, hdr, smem_raw, blockIdx.x, gridDim.x);
+  page_body<false, false>(L, hdr, smem_raw, blockIdx.x, gridDim.x, 0);
+}
+
+// The page pass over the units' slot lists (list pass `which`).
+__global__ void __launch_bounds__(512, 1) pass_b_list_tc(const __grid_constant__ TcLaunch L, WsHeader *hdr, int which) {
+  extern __shared__ uint8_t smem_raw[];
+  const int n = L.n_list_items[which];
+  if ((int)blockIdx.x >= n) return;
+  page_body<false, true>(L, hdr, smem_raw, blockIdx.x, gridDim.x, n);
+}
+
+// ============================================================== bounds and lists
+// R(E) is a maximum over units and rows (Eq. 7), so a unit whose effects
+// cannot exceed a value of R(E) that is already there need not score page E.
+// With s the page's share of the row's attention,
+//   r = ||U_E - S_E o|| / ((l - S_E) ||o||)  <=  s / (1 - s) (1 + max|v| / ||o||)
+// since ||U_E|| <= S_E max|v|.  The flash pass leaves log2 S_E (rounded up)
+// of every row and page and |v| of every token; this kernel takes the
+// maximum of the bound over the unit's rows.  Shares above 0.9, where
+// rounding in l - S_E matters, rows with an output norm that is not an
+// ordinary number, and NaN give an infinite bound; the factors cover the
+// rounding of the terms.
+constexpr int kBoundPages = 64;  // pages per block: eight consecutive ones per warp
+__global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLaunch L) {
+  const int t = traj_of(L.bound_off, L.n_traj, blockIdx.x);
+  const TcTraj &tr = L.t[t];
+  const TcPrune &pr = tr.pr;
+  const int npb = (tr.P + kBoundPages - 1) / kBoundPages, local = blockIdx.x - L.bound_off[t];
+  const int unit = local / npb, rt = unit % tr.nrt, slice = unit / tr.nrt;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  constexpr int kPer = kBoundPages / 8;
+  const int Ew = local % npb * kBoundPages + warp * kPer, np = min(kPer, tr.P - Ew);
+  if (np <= 0) return;
+  const __half *pieces = pr.pieces + (int64_t)unit * pr.npiece * BM + 4 * lane;  // lane i: rows 4 i .. 4 i + 3
+  const __half *vn = pr.vnorm + (int64_t)slice * ((tr.S + BT - 1) / BT * BT);
+  auto load = [&](int piece) { return __ldg(reinterpret_cast<const uint2 *>(pieces + (int64_t)piece * BM)); };
+  // lane i reads page i's table entries; the loads of all pages are issued
+  // before any is used
+  const int po_l = pr.piece_off[Ew + min(lane, np)];
+  const int ps_l = tr.ps[Ew + min(lane, np - 1)], pl_l = tr.pl[Ew + min(lane, np - 1)];
+  uint2 w0[kPer], w1[kPer];
+  unsigned short v0[kPer];
+  const uint2 none = make_uint2(0xfc00fc00u, 0xfc00fc00u);  // -inf: no mass
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int p0 = __shfl_sync(0xffffffffu, po_l, i), p1 = __shfl_sync(0xffffffffu, po_l, i + 1);
+    const int b = __shfl_sync(0xffffffffu, ps_l, i), n = __shfl_sync(0xffffffffu, pl_l, i);
+    const bool any = i < np && p1 > p0;
+    w0[i] = any ? load(p0) : none;
+    w1[i] = any && p1 > p0 + 1 ? load(p0 + 1) : none;
+    v0[i] = any && lane < n ? __half_as_ushort(vn[b + lane]) : (unsigned short)0;
+  }
+  float m2[4], inv_l[4], inv_o[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool ok = rt * BM + 4 * lane + k < L.g * tr.W;
+    const float4 a = ok ? pr.aux[(int64_t)unit * BM + 4 * lane + k] : make_float4(-INFINITY, 0.0f, 1.0f, 0.0f);
+    const bool live = a.x != -INFINITY;  // the row sees something
+    m2[k] = live ? a.x - (1e-3f + 1e-6f * fabsf(a.x)) : INFINITY;
+    inv_l[k] = live ? 1.002f / a.y : 0.0f;
+    inv_o[k] = !live ? 0.0f : a.z > 1e-15f && a.z < 1e30f ? 1.01f / a.z : INFINITY;
+  }
+  auto add = [&](float (&S)[4], uint2 w) {
+    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
+    const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&w.y));
+    S[0] += fast_exp2(a.x - m2[0]);
+    S[1] += fast_exp2(a.y - m2[1]);
+    S[2] += fast_exp2(b.x - m2[2]);
+    S[3] += fast_exp2(b.y - m2[3]);
+  };
+  unsigned mine = 0;  // lane i: the bound of page i
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int p0 = __shfl_sync(0xffffffffu, po_l, i), p1 = __shfl_sync(0xffffffffu, po_l, i + 1);
+    const int b = __shfl_sync(0xffffffffu, ps_l, i), n = __shfl_sync(0xffffffffu, pl_l, i);
+    unsigned vb = v0[i];
+    float S[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    add(S, w0[i]);
+    add(S, w1[i]);
+    if (i < np && p1 > p0) {  // pages of more than 32 tokens, or more than two tiles
+      for (int k = lane + 32; k < n; k += 32) vb = max(vb, (unsigned)__half_as_ushort(vn[b + k]));
+      for (int p = p0 + 2; p < p1; ++p) add(S, load(p));
+    }
+    const float v = __half2float(__ushort_as_half((unsigned short)__reduce_max_sync(0xffffffffu, vb)));
+    unsigned mx = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float s = S[k] * inv_l[k];
+      float r = __fdividef(s, 1.0f - s) * (1.0f + v * inv_o[k]);
+      if (m2[k] == INFINITY) r = 0.0f;
+      else if (!(s < 0.9f) || !(r >= 0.0f)) r = INFINITY;
+      mx = max(mx, __float_as_uint(r));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == i) mine = mx;
+  }
+  if (lane < np) pr.bound[(int64_t)unit * tr.P + Ew + lane] = __uint_as_float(mine);
+}
+
+// Per page the unit with the largest bound: a block takes 32 pages, its
+// warps the units in turn.
+__global__ void __launch_bounds__(512) seed_kernel(const __grid_constant__ TcLaunch L) {
+  const int t = traj_of(L.seed_off, L.n_traj, blockIdx.x);
+  const TcTraj &tr = L.t[t];
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int E = (blockIdx.x - L.seed_off[t]) * 32 + lane, units = L.unit_off[t + 1] - L.unit_off[t];
+  __shared__ unsigned long long s_key[16][32];
+  unsigned long long key = 0ull;
+  if (E < tr.P && tr.slot_off[E + 1] > tr.slot_off[E])
+    for (int u = warp; u < units; u += 16) {
+      const unsigned b = __float_as_uint(tr.pr.bound[(int64_t)u * tr.P + E]);  // non-negative, infinite or NaN
+      const unsigned long long k = ((unsigned long long)b << 32) | (unsigned)u;
+      if (b != 0u && k > key) key = k;
+    }
+  s_key[warp][lane] = key;
+  __syncthreads();
+  if (warp == 0 && E < tr.P) {
+    for (int w = 1; w < 16; ++w) key = key > s_key[w][lane] ? key : s_key[w][lane];
+    tr.pr.seed[E] = key;
+  }
+}
+
+// Writes the slot list of one unit per block and its work items.  Pass 0
+// takes the pages whose seed this unit is; pass 1, when R holds the seeds'
+// effects, the other pages whose bound is above R.  A page whose bound is 0
+// has no visible mass and effect 0.  Items: item k of a unit takes the pages
+// whose first slot in its list lies in [k n, (k + 1) n).
+constexpr int kMaxBuckets = 1024;
+__global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLaunch L, int which) {
+  const int t = traj_of(L.unit_off, L.n_traj, blockIdx.x);
+  const TcTraj &tr = L.t[t];
+  const TcPrune &pr = tr.pr;
+  const int unit = blockIdx.x - L.unit_off[t];
+  const int per = max(kListSlotsPerItem, (pr.cap + kMaxBuckets - 1) / kMaxBuckets);
+  const int nbuckets = (pr.cap + per - 1) / per;
+  __shared__ unsigned long long s_first[kMaxBuckets];  // {first list entry, first page} of every bucket
+  __shared__ unsigned long long s_warp[8], s_run;
+  __shared__ int s_n, s_at;
+  for (int i = threadIdx.x; i < nbuckets; i += 256) s_first[i] = ~0ull;
+  if (threadIdx.x == 0) s_run = 0ull, s_n = 0;
+  __syncthreads();
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  int32_t *list = pr.list + (int64_t)unit * pr.cap;
+  for (int c0 = 0; c0 < tr.P; c0 += 256) {
+    const int E = c0 + threadIdx.x;
+    bool take = false;
+    int s0 = 0, ns = 0;
+    if (E < tr.P) {
+      s0 = tr.slot_off[E];
+      ns = tr.slot_off[E + 1] - s0;
+      const bool mine = pr.seed[E] != 0ull && (unsigned)(pr.seed[E] & 0xffffffffull) == (unsigned)unit;
+      if (which == 0) take = mine;
+      else {
+        const float b = pr.bound[(int64_t)unit * tr.P + E];
+        take = !mine && b != 0.0f && !(b <= tr.R[E]);
+      }
+      take = take && ns > 0;
+    }
+    // running (slots, pages taken) before this page
+    const unsigned long long v = take ? ((unsigned long long)1 << 32) | (unsigned)ns : 0ull;
+    unsigned long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    unsigned long long excl = s_run + x - v, total = 0ull;
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) excl += s_warp[w];
+      total += s_warp[w];
+    }
+    if (take) {
+      const int off = (int)(excl & 0xffffffffull), page = (int)(excl >> 32);
+      for (int k = 0; k < ns; ++k) list[off + k] = s0 + k;
+      atomicMin(&s_first[off / per], ((unsigned long long)off << 32) | (unsigned)page);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_run += total;
+    __syncthreads();
+  }
+  const unsigned long long all = ((s_run & 0xffffffffull) << 32) | (s_run >> 32);  // {slots, pages}
+  for (int i = threadIdx.x; i < nbuckets; i += 256)
+    if (s_first[i] != ~0ull) atomicAdd(&s_n, 1);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_at = s_n ? atomicAdd(&L.n_list_items[which], s_n) : 0;
+    s_n = 0;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nbuckets; i += 256) {
+    const unsigned long long a = s_first[i];
+    if (a == ~0ull) continue;
+    unsigned long long e = all;
+    for (int j = i + 1; j < nbuckets; ++j)
+      if (s_first[j] != ~0ull) {
+        e = s_first[j];
+        break;
+      }
+    const int off = (int)(a >> 32), nslot = (int)(e >> 32) - off;
+    const int npages = (int)(e & 0xffffffffull) - (int)(a & 0xffffffffull);
+    L.list_items[s_at + atomicAdd(&s_n, 1)] = make_int4((int)blockIdx.x, off, nslot, npages);
+  }
 }
 
 // ============================================================== fused
@@ -1401,8 +1846,8 @@ __global__ void __launch_bounds__(512, 1) pass_b_tc(const __grid_constant__ TcLa
 // they are still in L2.  Every cross-CTA wait is bounded.
 __global__ void __launch_bounds__(512, 1) score_fused_tc(const __grid_constant__ TcLaunch L, WsHeader *hdr) {
   extern __shared__ uint8_t smem_raw[];
-  if ((int)blockIdx.x < L.n_a) flash_body<true>(L, hdr, smem_raw, blockIdx.x, L.n_a);
-  else page_body<true>(L, hdr, smem_raw, blockIdx.x - L.n_a, gridDim.x - L.n_a);
+  if ((int)blockIdx.x < L.n_a) flash_body<true, false>(L, hdr, smem_raw, blockIdx.x, L.n_a);
+  else page_body<true, false>(L, hdr, smem_raw, blockIdx.x - L.n_a, gridDim.x - L.n_a, 0);
 }
 
 
@@ -1446,6 +1891,61 @@ bool map_kv(CUtensorMap *m, const void *base, int S, int H, int M, int64_t st, i
 }
 
 }  // namespace
+
+namespace {
+struct PruneSizes {
+  size_t cuts, tile, piece_off, pieces, vnorm, aux, bound, seed, list;
+  int npiece, cap;
+};
+PruneSizes prune_sizes(int S, int P, int slices, int nrt) {
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t ntile = ((size_t)S + BT - 1) / BT, units = (size_t)slices * nrt;
+  const size_t p = (size_t)(P < S / kMinPageTokens ? P : S / kMinPageTokens);
+  PruneSizes z;
+  z.npiece = (int)(p + ntile);
+  z.cap = (int)((size_t)S / SLOT + 1 + p);
+  z.cuts = up(4 * ntile * sizeof(uint2));
+  z.tile = up(ntile * sizeof(int2));
+  z.piece_off = up((p + 1) * 4);
+  z.pieces = up(units * z.npiece * BM * sizeof(__half));
+  z.vnorm = up((size_t)slices * ntile * BT * sizeof(__half));
+  z.aux = up(units * BM * sizeof(float4));
+  z.bound = up(units * p * 4);
+  z.seed = up(p * 8);
+  z.list = up(units * z.cap * 4);
+  return z;
+}
+}  // namespace
+
+size_t prune_bytes(int S, int P, int slices, int nrt) {
+  const PruneSizes z = prune_sizes(S, P, slices, nrt);
+  return z.cuts + z.tile + z.piece_off + z.pieces + z.vnorm + z.aux + z.bound + z.seed + z.list;
+}
+
+size_t prune_item_bytes(int S, int P, int slices, int nrt) {
+  const PruneSizes z = prune_sizes(S, P, slices, nrt);
+  return (size_t)slices * nrt * ((size_t)z.cap / kListSlotsPerItem + 1) * sizeof(int4);
+}
+
+void prune_layout(TcPrune &p, char *base, int S, int P, int slices, int nrt) {
+  const PruneSizes z = prune_sizes(S, P, slices, nrt);
+  auto take = [&](size_t n) {
+    char *at = base;
+    base += n;
+    return at;
+  };
+  p.cuts = reinterpret_cast<uint2 *>(take(z.cuts));
+  p.tile = reinterpret_cast<int2 *>(take(z.tile));
+  p.piece_off = reinterpret_cast<int32_t *>(take(z.piece_off));
+  p.pieces = reinterpret_cast<__half *>(take(z.pieces));
+  p.vnorm = reinterpret_cast<__half *>(take(z.vnorm));
+  p.aux = reinterpret_cast<float4 *>(take(z.aux));
+  p.bound = reinterpret_cast<float *>(take(z.bound));
+  p.seed = reinterpret_cast<unsigned long long *>(take(z.seed));
+  p.list = reinterpret_cast<int32_t *>(take(z.list));
+  p.npiece = z.npiece;
+  p.cap = z.cap;
+}
 
 size_t smem_a() { return sizeof(SmemA) + 1024; }
 size_t smem_b() { return sizeof(SmemB) + 1024; }
@@ -1516,14 +2016,34 @@ cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t s, int sm_c
     void *args[] = {(void *)&L, (void *)&hdr};
     return cudaLaunchCooperativeKernel((const void *)score_fused_tc, dim3(L.n_a + nb), dim3(512), args, smem, s);
   }
-  e = cudaFuncSetAttribute(pass_a_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a());
+  const auto pass_a = L.prune ? pass_a_tc<true> : pass_a_tc<false>;
+  e = cudaFuncSetAttribute(pass_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a());
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(pass_b_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b());
+  e = L.prune ? cudaFuncSetAttribute(pass_b_list_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b())
+              : cudaFuncSetAttribute(pass_b_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b());
   if (e != cudaSuccess) return e;
+  if (L.prune) {
+    L.bound_off[0] = L.seed_off[0] = 0;
+    for (int t = 0; t < L.n_traj; ++t) {
+      const int units = L.unit_off[t + 1] - L.unit_off[t], P = units > 0 ? L.t[t].P : 0;
+      L.bound_off[t + 1] = L.bound_off[t] + units * ((P + kBoundPages - 1) / kBoundPages);
+      L.seed_off[t + 1] = L.seed_off[t] + (P + 31) / 32;
+    }
+  }
   prep_kernel<<<L.n_traj, 1024, 0, s>>>(L, hdr);
-  if (na_items > 0) pass_a_tc<<<na_items < sm_count ? na_items : sm_count, 384, smem_a(), s>>>(L, hdr);
+  if (na_items > 0) pass_a<<<na_items < sm_count ? na_items : sm_count, L.prune ? 512 : 384, smem_a(), s>>>(L, hdr);
   const int rows = L.from_stats ? 0 : L.row_off[L.n_traj];
   if (rows > 0) combine_tc<<<(rows * 32 + 255) / 256, 256, 0, s>>>(L);
+  if (L.prune) {
+    const int units = L.unit_off[L.n_traj];
+    bound_kernel<<<L.bound_off[L.n_traj], 256, 0, s>>>(L);
+    seed_kernel<<<L.seed_off[L.n_traj], 512, 0, s>>>(L);
+    for (int which = 0; which < 2; ++which) {
+      list_kernel<<<units, 256, 0, s>>>(L, which);
+      pass_b_list_tc<<<sm_count, 512, smem_b(), s>>>(L, hdr, which);
+    }
+    return cudaGetLastError();
+  }
   if (nb_items > 0) pass_b_tc<<<nb_items < sm_count ? nb_items : sm_count, 512, smem_b(), s>>>(L, hdr);
   return cudaGetLastError();
 }

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_fp16.h>
 
 #include "ckv_internal.cuh"
 
@@ -27,20 +28,39 @@ struct TcMaps {
 // Per-trajectory facts computed once per call by the prep kernel.
 struct TcPrep {
   int vis_all;  // leading resident tokens visible to every probe row
-  int pad[3];
+  int nitem;    // entries of the item table that hold pages
+  int pad[2];
+};
+
+// A unit is one 128-row tile of probe rows of one (trajectory, selected
+// layer, KV head) slice: unit (li * H + kvh) * nrt + rt of its trajectory.
+// Workspace of the pruned page pass, per trajectory; null pointers when the
+// launch is not pruned.
+struct TcPrune {
+  uint2 *cuts;         // [4 ntile]: per 32 tokens, {page starts and ends, page ends} as bit masks
+  int2 *tile;          // [ntile]: {index of the tile's first piece, 1 if a page covers its last token}
+  int32_t *piece_off;  // [P + 1]: first piece of every page (a page has one piece per tile it touches)
+  __half *pieces;      // [units][npiece][128]: log2 of the row's exp-sum over the piece, rounded up
+  __half *vnorm;       // [slices][128 ntile]: upper bound of every token's |v|
+  float4 *aux;         // [units][128]: {final max (base 2), exp-sum, |o|, 0} of every probe row
+  float *bound;        // [units][P]: upper bound of the page's effect on the unit's rows
+  unsigned long long *seed;  // [P]: {bound bits, unit} of the unit with the largest bound (0: no effect)
+  int32_t *list;       // [units][cap]: slots of the unit's pages that are to be scored
+  int npiece, cap;
 };
 
 struct TcTraj {
   const int32_t *pos, *qpos, *ps, *pl;
   int32_t *slot_off;  // workspace [P + 1]
   int4 *items;        // workspace [nbitem][2]: {E0, E1, slot0, nslot}, {npages, 0, 0, 0}
-  int4 *slot_tab;     // workspace [ceil(S/16) + P]: {tok0, nv, page, first | last << 1 | rank << 2}
+  int4 *slot_tab;     // workspace [ceil(S/16) + P]: {tok0, nv, page, first | last << 1}
   TcPrep *prep;       // workspace
   int32_t *nvis_w;    // workspace [W]: resident tokens visible to each window position
   float *stats;       // [M][Hq][W][132]
   float *R;           // [P]
   float *headR;       // [M][Hq][P] or null
   int S, W, P, nchunk, nrt, nbitem;
+  TcPrune pr;
 };
 
 struct TcLaunch {
@@ -57,8 +77,35 @@ struct TcLaunch {
   int slice_off[kMaxTc + 1];  // (trajectory, selected layer, KV head) slices: prefix per trajectory
   uint32_t *a_done;           // workspace [slices][kCounterStride]: flash-pass warps done with their partials
   uint32_t *merged;           // workspace [slices][kCounterStride]: merge warps done with their rows
+  // pruned page pass (set by the caller): only the pages of a unit whose
+  // bound can raise R are scored
+  int prune;
+  int unit_off[kMaxTc + 1];   // units: prefix per trajectory
+  int bound_off[kMaxTc + 1];  // blocks of bound_kernel: prefix per trajectory
+  int seed_off[kMaxTc + 1];   // blocks of seed_kernel
+  int4 *list_items;           // workspace: {unit, first entry of its list, entries, pages} of every work item
+  int *n_list_items;          // workspace [2]: items of the two list passes
   uint8_t layer_ids[kMaxLayers];
 };
+
+// Bytes of workspace of the pruned page pass for one trajectory of up to S
+// tokens and P pages (monotone in S, P, slices and nrt), and of the shared
+// part (list_items) that it adds.
+size_t prune_bytes(int S, int P, int slices, int nrt);
+size_t prune_item_bytes(int S, int P, int slices, int nrt);
+// Lays the region out at `base`.
+void prune_layout(TcPrune &p, char *base, int S, int P, int slices, int nrt);
+// The page pass is pruned when the pages average at least kMinPageTokens
+// tokens (bounds the bookkeeping, which is per page and row: with 36 layers,
+// 8 KV heads and 16K + 2K tokens the call takes 6.0 ms against 15.5 ms with
+// the full pass for pages of 2 tokens, 1.53 against 2.28 ms for 32, 1.76
+// against 2.05 ms for 256), and when the launch has kMinPruneWork (unit,
+// token) pairs: below, the extra launches cost more than they save (1 layer
+// of 16K + 2K tokens 180 against 133 us, 36 layers of 1.5K tokens 432 against
+// 390 us; 4 layers of 16K + 2K 308 against 354 us, 36 layers of 4K 674
+// against 855 us).
+constexpr int kMinPageTokens = 2;
+constexpr int64_t kMinPruneWork = 1 << 20;
 
 size_t smem_a();
 size_t smem_b();

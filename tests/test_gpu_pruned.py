@@ -1,0 +1,121 @@
+"""The pruned page pass scores only the (unit, page) pairs whose bound can
+raise R, with the arithmetic of the full page pass: R is the same number,
+bit for bit.  The full pass runs when maxima per head are asked for."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_07855_gb300 import commitkv as ck
+
+pytestmark = pytest.mark.gpu
+
+
+def _pages(S, rng, sizes, gap):
+    ps, pl, t = [], [], int(rng.integers(0, 40))
+    while True:
+        n = int(rng.choice(sizes))
+        if t + n > S:
+            break
+        ps.append(t)
+        pl.append(n)
+        t += n + (int(rng.integers(0, gap + 1)) if rng.random() < 0.3 else 0)
+    return ps, pl
+
+
+def _traj(M, H, Hq, d, S, W, sizes, kind, seed, gap=60):
+    gen = torch.Generator("cuda").manual_seed(seed)
+    rng = np.random.default_rng(seed)
+
+    def normal(*s):
+        return torch.randn(*s, generator=gen, device="cuda")
+
+    K, V, Q = normal(M, H, S, d), normal(M, H, S, d), normal(M, Hq, W, d)
+    if kind == "sharp":  # a few tokens hold nearly all of some rows' attention
+        K[:, :, :: max(S // 7, 1)] *= 6.0
+    elif kind == "uniform":  # every share alike: no bound is far from the effect
+        K.zero_()
+    elif kind == "zero_v":
+        V.zero_()
+    elif kind == "small":  # squares of the values underflow
+        V *= 1e-21
+    elif kind == "big_v":  # norms above the range of 16-bit floats
+        V *= 3e5
+    elif kind == "inf_v":
+        V[0, 0, S // 2] = float("inf")
+    elif kind == "nan_k":
+        K[M - 1, 0, S // 3, 0] = float("nan")
+    pos = torch.cumsum(torch.randint(1, 3, (S,), generator=gen, device="cuda"), 0).int()
+    last = int(pos[-1])
+    qpos = torch.arange(last - W + 1, last + 1, dtype=torch.int32, device="cuda")
+    if kind == "blind":  # the first window position sees nothing
+        qpos[0] = -5
+    ps, pl = _pages(S, rng, sizes, gap)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    return ck.TrajTensors(K.bfloat16(), V.bfloat16(), pos, Q.bfloat16(), qpos, torch.tensor(ps, **i32),
+                          torch.tensor(pl, **i32))
+
+
+CASES = [
+    # M, H, Hq, W, S, page sizes, kind; each over the amount of work from which the page pass is pruned
+    (64, 8, 32, 16, 2100, [32], "normal"),
+    (64, 8, 32, 32, 2113, [16], "sharp"),
+    (64, 8, 64, 20, 1500, [8, 9, 127, 128, 129, 300], "normal"),  # 160 rows: a ragged second row tile
+    (64, 8, 16, 8, 2200, [0, 32, 33], "sharp"),
+    (128, 8, 32, 16, 1100, [32], "uniform"),
+    (256, 16, 32, 32, 300, [16], "zero_v"),
+    (256, 8, 16, 8, 513, [16, 40], "small"),
+    (256, 8, 16, 8, 512, [64], "big_v"),
+    (128, 8, 16, 8, 1100, [32], "inf_v"),
+    (128, 8, 16, 8, 1100, [32], "nan_k"),
+    (256, 8, 16, 4, 600, [32], "blind"),
+    (64, 8, 16, 4, 3000, [2800], "sharp"),  # one page of many tiles holding almost everything
+    (64, 8, 16, 8, 2100, [2, 3], "normal"),
+    (64, 8, 16, 8, 2100, [1, 2], "normal"),  # pages too short to prune: the full pass both times
+]
+
+
+def _both(trajs, M, Hq, mask=None):
+    shape = ck.make_shape(M, trajs[0].k.shape[1], Hq, 128, torch.bfloat16)
+    ws = ck.alloc_workspace(shape, trajs)
+    out = []
+    for head in (False, True):
+        R = [torch.full((t.page_start.numel(),), -1.0, device="cuda") for t in trajs]
+        hR = [torch.zeros(M, Hq, t.page_start.numel(), device="cuda") for t in trajs] if head else None
+        ck.commitkv_page_effects(shape, trajs, R, head_R_out=hR, layer_mask=mask, workspace=ws)
+        assert ck.commitkv_workspace_status(ws) == ck.COMMITKV_OK
+        out.append([r.cpu().numpy().view(np.uint32) for r in R])
+    return out
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[6]}-{c[4]}-{c[5][0]}")
+def test_pruned_effects_equal_the_full_pass(case):
+    M, H, Hq, W, S, sizes, kind = case
+    for seed in (1, 2):
+        pruned, full = _both([_traj(M, H, Hq, 128, S, W, sizes, kind, seed)], M, Hq)
+        assert np.array_equal(pruned[0], full[0])
+
+
+def test_pruned_effects_of_a_ragged_batch_with_a_layer_mask():
+    sizes = [300, 2000, 129, 777, 1300]
+    trajs = [_traj(256, 2, 8, 128, S, W, [16, 32], "sharp", i) for i, (S, W) in enumerate(zip(sizes, [8, 32, 4, 40, 16]))]
+    none = torch.zeros(0, dtype=torch.int32, device="cuda")
+    trajs.append(ck.TrajTensors(trajs[0].k, trajs[0].v, trajs[0].pos, trajs[0].q, trajs[0].q_pos, none, none))
+    for mask in (None, [0, 1] * 128):
+        pruned, full = _both(trajs, 256, 8, mask)
+        for a, b in zip(pruned, full):
+            assert np.array_equal(a, b)
+
+
+def test_overlapping_pages_are_reported_and_stay_in_bounds():
+    """A zero-length page between two pages of the same span: each is
+    compared with every earlier page, not with its neighbour alone."""
+    t = _traj(128, 8, 16, 128, 1100, 8, [32], "normal", 3)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    t.page_start = torch.tensor([0, 0, 0, 0, 0, 1080], **i32)
+    t.page_len = torch.tensor([1000, 0, 1000, 0, 1000, 12], **i32)
+    shape = ck.make_shape(128, 8, 16, 128, torch.bfloat16)
+    ws = ck.alloc_workspace(shape, [t])
+    for head in (None, [torch.zeros(128, 16, 6, device="cuda")]):
+        R = torch.zeros(6, device="cuda")
+        ck.commitkv_page_effects(shape, [t], [R], head_R_out=head, workspace=ws)
+        assert ck.commitkv_workspace_status(ws) == ck.COMMITKV_ERR_DEVICE_INPUT
