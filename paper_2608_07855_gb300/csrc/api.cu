@@ -133,7 +133,7 @@ int chunk_len_for(int n_traj, const commitkv_traj *tr) {
 
 int cdiv(int a, int b) { return (a + b - 1) / b; }
 
-// ---- tensor-core scoring path (bf16, head_dim 128)
+// ---- tensor-core scoring path (bf16)
 int tc_chunk_len(int n_traj, const commitkv_traj *tr) {
   int smax = 0;
   for (int t = 0; t < n_traj; ++t) smax = tr[t].S > smax ? tr[t].S : smax;
@@ -161,7 +161,7 @@ bool env_force_simt() {
 }
 
 bool tc_eligible(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
-  if (s->dtype != COMMITKV_BF16 || s->head_dim != 128 || env_force_simt()) return false;
+  if (s->dtype != COMMITKV_BF16 || env_force_simt()) return false;
   for (int t = 0; t < n_traj; ++t) {
     const commitkv_traj &x = tr[t];
     if (x.S == 0 || x.W == 0 || x.P == 0) continue;
@@ -233,7 +233,7 @@ size_t tc_score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *
              align_up(tc::prune_item_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt)) + kAlign;
     slices += (size_t)s->layers * s->kv_heads;
   }
-  return align_up(tc_partial_slots(s, n_traj, tr) * tc::kPartsPerItem * tc::kRowsPerTile * 132 * 4) +
+  return align_up(tc_partial_slots(s, n_traj, tr) * tc::kPartsPerItem * tc::kRowsPerTile * (s->head_dim + 4) * 4) +
          align_up(slices * 2 * tc::kCounterStride * 4) + slots;
 }
 
@@ -249,10 +249,8 @@ size_t score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr,
     stats += align_up((size_t)s->layers * s->q_heads * tr[t].W * (d + 4) * 4) + align_up((size_t)tr[t].W * 4);
   }
   size_t scratch = align_up(units * RB * (d + 4) * 4);
-  if (s->head_dim == 128) {
-    size_t tcb = tc_score_bytes(s, n_traj, tr);
-    if (tcb > scratch) scratch = tcb;
-  }
+  const size_t tcb = tc_score_bytes(s, n_traj, tr);
+  if (tcb > scratch) scratch = tcb;
   return scratch + stats;
 }
 
@@ -389,10 +387,8 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   for (int t = 0; t < n_traj; ++t)
     full_units += (size_t)shape->layers * shape->kv_heads * simt_chunk_bound(trajs[t].S) * L.nrb[t];
   size_t scratch = align_up(full_units * RB * (d + 4) * 4);
-  if (shape->head_dim == 128) {
-    size_t tcb = tc_score_bytes(shape, n_traj, trajs);
-    if (tcb > scratch) scratch = tcb;
-  }
+  const size_t tcb = tc_score_bytes(shape, n_traj, trajs);
+  if (tcb > scratch) scratch = tcb;
   char *sbase = base + scratch;
   for (int t = 0; t < n_traj; ++t) {
     size_t sb = align_up((size_t)shape->layers * shape->q_heads * trajs[t].W * (d + 4) * 4);
@@ -422,7 +418,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_status(e);
-  const bool fused = !from_stats && env_fused();
+  const bool fused = !from_stats && env_fused() && d == 128;
   int CLt = tc_chunk_len(n_traj, trajs);
   if (fused) {
     int smax = 0, nrt_max = 1;
@@ -437,7 +433,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   size_t slices_all = 0;
   for (int t = 0; t < n_traj; ++t) slices_all += (size_t)shape->layers * shape->kv_heads;
   char *cnt_base = base + align_up(tc_partial_slots(shape, n_traj, trajs) * tc::kPartsPerItem * tc::kRowsPerTile *
-                                   132 * 4);
+                                   (d + 4) * 4);
   char *slot_base = cnt_base + align_up(slices_all * 2 * tc::kCounterStride * 4);
   for (int b0 = 0; b0 < n_traj; b0 += tc::kMaxTc) {
     int nb = n_traj - b0 < tc::kMaxTc ? n_traj - b0 : tc::kMaxTc;
@@ -501,7 +497,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       T.row_off[i + 1] = T.row_off[i] + (active ? nl * shape->kv_heads * L.batch.g * x.W : 0);
       T.slice_off[i + 1] = T.slice_off[i] + (active ? nl * shape->kv_heads : 0);
       T.unit_off[i + 1] = T.unit_off[i] + (active && x.P > 0 ? nl * shape->kv_heads * c.nrt : 0);
-      if (active && !tc::build_maps(T.maps[i], L.batch.t[t], shape->layers, shape->kv_heads, shape->q_heads))
+      if (active && !tc::build_maps(d, T.maps[i], L.batch.t[t], shape->layers, shape->kv_heads, shape->q_heads))
         return COMMITKV_ERR_CUDA;
     }
     // one array of work items for the launch, after its trajectories' regions
@@ -509,7 +505,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     for (int i = 0; i < nb; ++i)
       slot_base += align_up(tc::prune_item_bytes(trajs[b0 + i].S, trajs[b0 + i].P, shape->layers * shape->kv_heads,
                                                  T.t[i].nrt));
-    e = tc::launch_score_tc(T, hdr, stream, sms);
+    e = tc::launch_score_tc(d, T, hdr, stream, sms);
     if (e != cudaSuccess) return cuda_status(e);
   }
   return COMMITKV_OK;

@@ -1,4 +1,4 @@
-// Launch description of the tensor-core scoring path (score_tc.cu).
+// Launch description of the tensor-core scoring path (score_tc_impl.cuh).
 #pragma once
 
 #include <cuda.h>
@@ -11,6 +11,9 @@ namespace tc {
 
 constexpr int kMaxTc = 16;          // trajectories per launch (tensor maps travel as parameters)
 constexpr int kRowsPerTile = 128;   // probe rows per MMA tile
+constexpr int kTileTokens = 128;    // tokens per MMA tile
+constexpr int kSlot = 16;           // tokens per page slot
+constexpr int kListSlotsPerItem = 64;  // slots per work item of the pruned page pass
 constexpr int kSlotsPerItem = 128;  // 16-token slots per pass-B work item
 constexpr int kPartsPerItem = 1;    // pass-A partials per work item (the two softmax groups merged)
 constexpr int kPartialRing = 4;     // partial slots (items) per flash CTA of the fused launch
@@ -20,8 +23,8 @@ constexpr double kFusedFlashShare = 0.55;  // share of the SMs that run the flas
 constexpr int kCounterStride = 32;  // per-slice counters of the fused launch, one 128-byte line each
 
 struct TcMaps {
-  CUtensorMap q;             // Q as [M*Hq*W rows][128], box 64 x 128
-  CUtensorMap k, v;          // K, V as [M][H][S][128], box 64 x 128 x 1 x 1
+  CUtensorMap q;             // Q as [M*Hq*W rows][d], box 64 x 128
+  CUtensorMap k, v;          // K, V as [M][H][S][d], box 64 x 128 x 1 x 1
   CUtensorMap kb[3], vb[3];  // the same with 16-, 32- and 64-row boxes (runs of page slots)
 };
 
@@ -56,7 +59,7 @@ struct TcTraj {
   int4 *slot_tab;     // workspace [ceil(S/16) + P]: {tok0, nv, page, first | last << 1}
   TcPrep *prep;       // workspace
   int32_t *nvis_w;    // workspace [W]: resident tokens visible to each window position
-  float *stats;       // [M][Hq][W][132]
+  float *stats;       // [M][Hq][W][d + 4]
   float *R;           // [P]
   float *headR;       // [M][Hq][P] or null
   int S, W, P, nchunk, nrt, nbitem;
@@ -69,7 +72,7 @@ struct TcLaunch {
   int n_traj, M, H, Hq, g, n_layers, chunk_len, slots_per_item;
   int from_stats;  // the stats are the caller's: no flash pass, no combine
   float scale_log2;
-  float *partials;  // [items_a or n_a * kPartialRing][2][128][132]: one partial per softmax warpgroup
+  float *partials;  // [items_a or n_a * kPartialRing][128][d + 4]: one partial per work item
   int item_off_a[kMaxTc + 1], item_off_b[kMaxTc + 1], row_off[kMaxTc + 1];
   // fused launch: CTAs [0, n_a) run the flash pass, the rest the page pass
   int fused;  // 1: one cooperative launch of both passes (set by the caller; needs !from_stats)
@@ -107,10 +110,21 @@ void prune_layout(TcPrune &p, char *base, int S, int P, int slices, int nrt);
 constexpr int kMinPageTokens = 2;
 constexpr int64_t kMinPruneWork = 1 << 20;
 
-size_t smem_a();
-size_t smem_b();
+// The kernels for one head width.
+namespace d128 {
 bool build_maps(TcMaps &maps, const TrajDev &t, int M, int H, int Hq);
 cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t stream, int sm_count);
+}  // namespace d128
+namespace d64 {
+bool build_maps(TcMaps &maps, const TrajDev &t, int M, int H, int Hq);
+cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t stream, int sm_count);
+}  // namespace d64
+inline bool build_maps(int d, TcMaps &maps, const TrajDev &t, int M, int H, int Hq) {
+  return d == 64 ? d64::build_maps(maps, t, M, H, Hq) : d128::build_maps(maps, t, M, H, Hq);
+}
+inline cudaError_t launch_score_tc(int d, TcLaunch &L, WsHeader *hdr, cudaStream_t stream, int sm_count) {
+  return d == 64 ? d64::launch_score_tc(L, hdr, stream, sm_count) : d128::launch_score_tc(L, hdr, stream, sm_count);
+}
 // Flash-pass CTAs of a fused launch on sm_count SMs (the rest run the page pass).
 int fused_flash_ctas(const TcLaunch &L, int sm_count);
 // Chunk length (tokens) of the fused launch for caches of up to max_tokens

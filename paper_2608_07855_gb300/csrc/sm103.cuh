@@ -259,6 +259,14 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
       "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15, %16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
 // Packed pair FMA: (a.x * b.x + c.x, a.y * b.y + c.y) in one instruction.
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   uint64_t d;
@@ -291,6 +299,24 @@ __device__ __forceinline__ void split_pack32(const float *x, uint32_t (&out)[32]
     __nv_bfloat162 l = __floats2bfloat162_rn(la, lb);
     out[e] = hi;
     out[16 + e] = *reinterpret_cast<uint32_t *>(&l);
+  }
+}
+
+// Takes one bf16 term off 32 fp32 values, packed two per 32-bit word: the
+// top 16 bits of x, which is left with the exact remainder, or, as the last
+// term, x rounded.  Three terms carry x to about 2^-25 relative.
+__device__ __forceinline__ void split_term32(float (&x)[32], uint32_t (&out)[16], bool last) {
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    if (last) {
+      __nv_bfloat162 l = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+      out[e] = *reinterpret_cast<uint32_t *>(&l);
+    } else {
+      uint32_t a = __float_as_uint(x[2 * e]), b = __float_as_uint(x[2 * e + 1]);
+      asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(out[e]) : "r"(a), "r"(b));
+      x[2 * e] -= __uint_as_float(a & 0xffff0000u);
+      x[2 * e + 1] -= __uint_as_float(b & 0xffff0000u);
+    }
   }
 }
 

@@ -403,7 +403,7 @@ cudaError_t launch_tc(const Batch &b, const float *const *stats, float *const *s
       tt.nchunk = (x.S + kTilesPerItem * BT - 1) / (kTilesPerItem * BT);
       const bool active = x.S > 0 && x.W > 0;
       L.item_off[i + 1] = L.item_off[i] + (active ? b.n_layers * b.H * tt.nchunk * tt.nrt : 0);
-      if (active && !tc::build_maps(L.maps[i], x, b.M, b.H, b.Hq)) return cudaErrorInvalidValue;
+      if (active && !tc::build_maps(D, L.maps[i], x, b.M, b.H, b.Hq)) return cudaErrorInvalidValue;
     }
     const int n = L.item_off[nb];
     if (n > 0) token_scores_tc<<<n < sm_count ? n : sm_count, 320, smem_bytes(), s>>>(L, hdr);
