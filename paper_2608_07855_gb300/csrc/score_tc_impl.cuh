@@ -4,8 +4,8 @@
 //
 //   pass A   persistent, warp-specialised flash forward over 128-token tiles
 //            of a token chunk: S = Q K^T (tcgen05, TMEM), online softmax in
-//            base 2 with a lazy max (O in TMEM is rescaled only when the row
-//            max grows by more than 2^8), O += P V (tcgen05); writes the
+//            base 2 with a lazy max (O is rescaled only when the row max
+//            grows by more than 2^8), O += P V; writes the
 //            chunk's (max, sum, count, O) per probe row.
 //   combine  merges a slice's chunk partials into the row stats
 //            (m, l, n, o) of the whole cache.
@@ -228,7 +228,7 @@ struct SmemA {
   float mused[2][BM];   // SUMS: per S/P buffer and row, the reference max of P
   float4 pub[BM];     // fused launch: warpgroup 1's (reference max, sum, count, true max) of the item, per row
   uint64_t q_full, q_empty, k_full[NKB], k_empty[NKB], v_full[NVB], v_empty[NVB], s_full[2], s_empty[2], p_full[2],
-      pv_done[2], o_full[2], o_empty[2], drain, drain2, pub_full, pub_empty;
+      o_full[2], o_empty[2], drain, drain2, pub_full, pub_empty;
   uint32_t tmem;
   int abort_flag;
 };
@@ -291,6 +291,20 @@ __device__ __forceinline__ void store_p(uint32_t buf, int c, float (&x)[32]) {
   }
 }
 
+// Two exponentials 2^(x scale + bias), the arguments in one instruction.
+__device__ __forceinline__ void exp2_pair(float *x, float2 scale, float2 bias) {
+  const float2 t = ffma2(make_float2(x[0], x[1]), scale, bias);
+  x[0] = fast_exp2(t.x);
+  x[1] = fast_exp2(t.y);
+}
+// Sum of eight values in packed pairs.
+__device__ __forceinline__ float sum8(const float *x) {
+  const float2 a = fadd2(make_float2(x[0], x[1]), make_float2(x[2], x[3]));
+  const float2 b = fadd2(make_float2(x[4], x[5]), make_float2(x[6], x[7]));
+  const float2 c = fadd2(a, b);
+  return c.x + c.y;
+}
+
 // log2 on the special-function unit (log2 0 = -inf).
 __device__ __forceinline__ float fast_log2(float x) {
   float y;
@@ -325,7 +339,6 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
       mbar_init(&sm.s_full[b], 1);
       mbar_init(&sm.s_empty[b], SUMS ? 5 : 1);
       mbar_init(&sm.p_full[b], 4);
-      mbar_init(&sm.pv_done[b], 1);
       mbar_init(&sm.o_full[b], 1);
       mbar_init(&sm.o_empty[b], 4);
     }
@@ -434,7 +447,6 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           for (int ks = 0; ks < BT / 16; ++ks) issue_pv_step(tm, 2 * PW + b * D, sm.v[s2], b, ks, (first || kRegO) && ks == 0);
           mma_commit(&sm.s_empty[b]);
           mma_commit(&sm.v_empty[s2]);
-          mma_commit(&sm.pv_done[b]);
           if (last) {
             mma_commit(&sm.o_full[b]);
             if (b) ++uses1;
@@ -503,6 +515,7 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
       int rows = L.g * tr.W;
       int grow = a.rt * BM + row;  // row within the (layer, KV head) slice
       bool valid_row = grow < rows;
+      const bool warp_rows = grow - lane < rows;  // the warp has a row of the slice
       int qp = valid_row ? tr.qpos[grow % tr.W] : -0x7fffffff;
       const int vis_all = tr.prep->vis_all;
       int t0 = a.c * L.chunk_len, t1 = min(tr.S, t0 + L.chunk_len);
@@ -542,13 +555,23 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           break;
         }
         tc_fence_after();
+        // A warp without a probe row of the slice leaves its rows as they are:
+        // rows are independent, and none of theirs is read.  (32 probe rows
+        // of 128, contexts of 2K tokens: flash pass 470 -> 232 us.)
+        if (!warp_rows) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.p_full[b]);
+          continue;
+        }
         // visibility of column i: inside the tile and, outside the prefix every
         // probe row sees, at or before the row's query position
-        const bool simple = full && nt == BT && valid_row;
-        // sweep 1: row max over the tile, 32 columns at a time
-        float mx[8];
+        const bool simple = full && nt == BT;
+        // row max over the tile, 32 columns at a time (the first sweep; the
+        // second computes P)
+        float mx[4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) mx[k] = -INFINITY;
+        for (int k = 0; k < 4; ++k) mx[k] = -INFINITY;
         int cnt = simple ? BT : 0;
 #pragma unroll 1
         for (int c0 = 0; c0 < BT; c0 += 32) {
@@ -558,7 +581,7 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           if (!simple) {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
-              bool vis = valid_row && c0 + i < nt && (full || posw[c0 + i] <= qp);
+              bool vis = c0 + i < nt && (full || posw[c0 + i] <= qp);
               x[i] = vis ? x[i] : -INFINITY;
               cnt += vis;
             }
@@ -566,9 +589,9 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
 #pragma unroll
           for (int i = 0; i < 32; i += 8)
 #pragma unroll
-            for (int k = 0; k < 8; ++k) mx[k] = fmaxf(mx[k], x[i + k]);
+            for (int k = 0; k < 4; ++k) mx[k] = fmax3(mx[k], x[i + 2 * k], x[i + 2 * k + 1]);
         }
-        float smax = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
+        float smax = fmaxf(fmax3(mx[0], mx[1], mx[2]), mx[3]);
         float mt = smax == -INFINITY ? smax : smax * L.scale_log2;
         nvis += cnt;
         m_true = fmaxf(m_true, mt);
@@ -577,12 +600,8 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
         float alpha = (rescale && m_used != -INFINITY) ? exp2f(m_used - m_new) : 0.0f;
         if (rescale) m_used = m_new;
         if (j > j0) {
-          // P V of this warpgroup's previous tile done: O_hb is stable
-          if (!__all_sync(0xffffffffu, mbar_wait(&sm.pv_done[b], ((g >> 1) - 1) & 1, kWait, abort_flag))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
+          // S of this tile is there, so the P V of this warpgroup's previous
+          // tile is done (Q K^T waited for the buffer): O_hb is stable
           if constexpr (kRegO) {
             take_o();
             if (rescale) {
@@ -591,7 +610,7 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
             }
           } else if (__any_sync(0xffffffffu, rescale)) {
             float f = rescale ? alpha : 1.0f;
-#pragma unroll
+#pragma unroll 1
             for (int c0 = 0; c0 < D; c0 += 32) {
               uint32_t r[32];
               tmem_ld32(tm + lane_base + o_col + c0, r);
@@ -605,8 +624,9 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
         }
         if (rescale) lsum *= alpha;
         const float neg_m = m_used == -INFINITY ? 0.0f : -m_used;
+        const float2 scale2 = make_float2(L.scale_log2, L.scale_log2), neg_m2 = make_float2(neg_m, neg_m);
         // sweep 2: p = 2^(s c - m) on the visible columns (2^-inf = 0), the row
-        // sum, and P as the (hi, lo) bf16 pair over the S columns just read
+        // sum, and P's terms over S columns already read
         float ps = 0.0f;
 #pragma unroll 1
         for (int c0 = 0; c0 < BT; c0 += 32) {
@@ -616,17 +636,15 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           if (!simple) {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
-              bool vis = valid_row && c0 + i < nt && (full || posw[c0 + i] <= qp);
+              bool vis = c0 + i < nt && (full || posw[c0 + i] <= qp);
               x[i] = vis ? x[i] : -INFINITY;
             }
           }
 #pragma unroll
-          for (int i = 0; i < 32; ++i) x[i] = fast_exp2(fmaf(x[i], L.scale_log2, neg_m));
+          for (int i = 0; i < 32; i += 2) exp2_pair(&x[i], scale2, neg_m2);
           float gs[4];  // sums of the four groups of eight columns
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            gs[q] = ((x[8 * q] + x[8 * q + 1]) + (x[8 * q + 2] + x[8 * q + 3])) +
-                    ((x[8 * q + 4] + x[8 * q + 5]) + (x[8 * q + 6] + x[8 * q + 7]));
+          for (int q = 0; q < 4; ++q) gs[q] = sum8(&x[8 * q]);
           ps += (gs[0] + gs[1]) + (gs[2] + gs[3]);
           if constexpr (SUMS) sm.gs[b][c0 / 32][row] = make_float4(gs[0], gs[1], gs[2], gs[3]);
           store_p(tm + lane_base + b * PW, c0 / 32, x);
@@ -768,6 +786,7 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           tr.pr.pieces + (int64_t)((a.li * L.H + a.kvh) * tr.nrt + a.rt) * tr.pr.npiece * BM + row;
       const int2 *tiles = tr.pr.tile + t0 / BT;
       const uint2 *cuts = tr.pr.cuts + t0 / 32;
+      const bool warp_rows = a.rt * BM + wq * 32 < L.g * tr.W;  // the warp has a probe row of the slice
 #pragma unroll 1
       for (int j = 0; j < ntile; ++j) {
         const uint32_t g = it + j;
@@ -786,6 +805,10 @@ __device__ __forceinline__ void flash_body(const TcLaunch &L, WsHeader *hdr, uin
           break;
         }
         tc_fence_after();
+        if (!warp_rows) {
+          if (lane == 0) mbar_arrive(&sm.s_empty[b]);
+          continue;
+        }
         __half *dst = piece_row + (int64_t)tile.x * BM;
         const float mu = sm.mused[b][row];
         // run: the row's sum before the chunk; base: before the segment being
@@ -1489,6 +1512,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
       int rows = L.g * tr.W;
       int grow = bi.rt * BM + row;
       bool valid_row = grow < rows;
+      const bool warp_rows = grow - lane < rows;  // a warp without a row of the slice only keeps the pages' order
       int qp = -0x7fffffff;
       // the row stats of this slice are complete once every share is merged
       if (FUSED && !warp_poll_geq(&L.merged[slice_of(L, bi)], 4u * items_per_slice(L, bi.t), abort_flag, hdr)) {
@@ -1539,35 +1563,32 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
         const int po_first = po_seen;
 #pragma unroll 1
         for (int ch = 0; ch < BT / 32 && ok; ++ch) {
-          float x[32];
-          // tensor-memory loads and stores are warp-collective: the lanes
-          // may have left the bounded waits above on different iterations
-          __syncwarp();
-          tmem_ld32f(tm + lane_base + b * PW + S0 + 32 * ch, x);
           const SlotMeta m0 = sm.meta[s][2 * ch], m1 = sm.meta[s][2 * ch + 1];
           uint32_t vm = (m0.nv >= SLOT ? 0xffffu : (1u << max(m0.nv, 0)) - 1u) |
                         ((m1.nv >= SLOT ? 0xffffu : (1u << max(m1.nv, 0)) - 1u) << 16);
-          if (!full) {
+          float s0 = 0.0f, s1 = 0.0f;
+          if (warp_rows) {
+            float x[32];
+            // tensor-memory loads and stores are warp-collective: the lanes
+            // may have left the bounded waits above on different iterations
+            __syncwarp();
+            tmem_ld32f(tm + lane_base + b * PW + S0 + 32 * ch, x);
+            if (!full) {
 #pragma unroll 1
-            for (int i = 0; i < 32; ++i)
-              if (sm.pos[wq][32 * ch + i] > qp) vm &= ~(1u << i);
-          }
-          if (!valid_row) vm = 0;
-          tmem_wait_ld();
-          float a0 = 0.f, a1 = 0.f, c0 = 0.f, c1 = 0.f;
+              for (int i = 0; i < 32; ++i)
+                if (sm.pos[wq][32 * ch + i] > qp) vm &= ~(1u << i);
+            }
+            if (!valid_row) vm = 0;
+            tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            float xi = (vm >> i) & 1u ? x[i] : -INFINITY;
-            x[i] = fast_exp2(fmaf(xi, L.scale_log2, neg_m2));
-          }
+            for (int i = 0; i < 32; ++i) x[i] = (vm >> i) & 1u ? x[i] : -INFINITY;
 #pragma unroll
-          for (int i = 0; i < 16; i += 2) {
-            a0 += x[i];
-            a1 += x[i + 1];
-            c0 += x[16 + i];
-            c1 += x[17 + i];
+            for (int i = 0; i < 32; i += 2)
+              exp2_pair(&x[i], make_float2(L.scale_log2, L.scale_log2), make_float2(neg_m2, neg_m2));
+            s0 = sum8(x) + sum8(x + 8);
+            s1 = sum8(x + 16) + sum8(x + 24);
+            store_p(tm + lane_base + b * PW, ch, x);
           }
-          store_p(tm + lane_base + b * PW, ch, x);
 #pragma unroll
           for (int h2 = 0; h2 < 2; ++h2) {
             const SlotMeta mt = h2 ? m1 : m0;
@@ -1576,7 +1597,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
               S_cur = 0.0f;
               n_cur = 0;
             }
-            S_cur += h2 ? c0 + c1 : a0 + a1;
+            S_cur += h2 ? s1 : s0;
             n_cur += __popc(h2 ? vm >> 16 : vm & 0xffffu);
             if (mt.flags & 2) {
               int f = po_seen % NFIFO;
@@ -1626,6 +1647,7 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
       int rows = L.g * tr.W;
       int grow = bi.rt * BM + row;
       bool valid_row = grow < rows;
+      const bool warp_rows = grow - lane < rows;
       int h = bi.kvh * L.g + (valid_row ? grow / tr.W : 0), w = valid_row ? grow % tr.W : 0;
       if (FUSED && !warp_poll_geq(&L.merged[slice_of(L, bi)], 4u * items_per_slice(L, bi.t), abort_flag, hdr)) {
         ok = false;
@@ -1668,6 +1690,13 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
         const float2 nS = make_float2(-S_E, -S_E);
         // ||U_E - S_E o||^2 over 16-column pieces of U_E
         float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+        if (!warp_rows) {  // no row of the slice: only hands the accumulator back
+          if (lane == 0) {
+            mbar_arrive(&sm.acc_empty[par]);
+            mbar_arrive(&sm.fifo_empty[f]);
+          }
+          continue;
+        }
 #pragma unroll
         for (int c0 = 0; c0 < D; c0 += 16) {
           uint32_t r[16];

@@ -277,6 +277,22 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return *reinterpret_cast<float2 *>(&d);
 }
 
+// Packed pair addition.
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(d)
+      : "l"(*reinterpret_cast<uint64_t *>(&a)), "l"(*reinterpret_cast<uint64_t *>(&b)));
+  return *reinterpret_cast<float2 *>(&d);
+}
+
+// The larger of three (a NaN is ignored, as by fmaxf).
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // 2^x on the special-function unit (PTX ex2.approx.ftz.f32; 2^-inf = 0).
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
@@ -294,9 +310,9 @@ __device__ __forceinline__ void split_pack32(const float *x, uint32_t (&out)[32]
     uint32_t a = __float_as_uint(x[2 * e]), b = __float_as_uint(x[2 * e + 1]);
     uint32_t hi;
     asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(hi) : "r"(a), "r"(b));
-    float la = x[2 * e] - __uint_as_float(a & 0xffff0000u);
-    float lb = x[2 * e + 1] - __uint_as_float(b & 0xffff0000u);
-    __nv_bfloat162 l = __floats2bfloat162_rn(la, lb);
+    const float2 r = ffma2(make_float2(__uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u)),
+                           make_float2(-1.0f, -1.0f), make_float2(x[2 * e], x[2 * e + 1]));  // exact
+    __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
     out[e] = hi;
     out[16 + e] = *reinterpret_cast<uint32_t *>(&l);
   }
@@ -314,8 +330,10 @@ __device__ __forceinline__ void split_term32(float (&x)[32], uint32_t (&out)[16]
     } else {
       uint32_t a = __float_as_uint(x[2 * e]), b = __float_as_uint(x[2 * e + 1]);
       asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(out[e]) : "r"(a), "r"(b));
-      x[2 * e] -= __uint_as_float(a & 0xffff0000u);
-      x[2 * e + 1] -= __uint_as_float(b & 0xffff0000u);
+      const float2 r = ffma2(make_float2(__uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u)),
+                             make_float2(-1.0f, -1.0f), make_float2(x[2 * e], x[2 * e + 1]));
+      x[2 * e] = r.x;
+      x[2 * e + 1] = r.y;
     }
   }
 }
