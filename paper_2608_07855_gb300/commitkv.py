@@ -130,15 +130,20 @@ def _check(rc: int, where: str):
 # marshalling helpers (torch tensors -> pointers)
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream(stream) -> Optional[int]:
-    torch = _torch()
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream or None
+        return _torch().cuda.current_stream().cuda_stream or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
@@ -155,15 +160,12 @@ def _ptr(x) -> Optional[int]:
 def _ptr_array(xs, n) -> Optional[ctypes.Array]:
     if xs is None:
         return None
-    arr = (ctypes.c_void_p * n)()
-    for i, x in enumerate(xs):
-        arr[i] = _ptr(x)
-    return arr
+    return (ctypes.c_void_p * n)(*map(_ptr, xs))
 
 
 def _require_cuda(*ts):
     for t in ts:
-        if t is not None and not isinstance(t, int) and t.numel() and not t.is_cuda:
+        if t is not None and not isinstance(t, int) and not t.is_cuda and t.numel():
             raise ValueError("CommitKV tensors must live on the GPU (no CPU fallback)")
 
 
@@ -182,20 +184,20 @@ class TrajTensors:
     page_len: object = None
 
     def desc(self) -> Traj:
-        torch = _torch()
-        k, v = self.k, self.v
-        _require_cuda(k, v, self.pos, self.q, self.q_pos, self.page_start, self.page_len)
-        assert k.dim() == 4 and k.stride() == v.stride() and k.shape == v.shape
-        assert k.stride(3) == 1, "head_dim must be contiguous"
-        for t in (self.pos, self.q_pos, self.page_start, self.page_len):
-            assert t is None or t.dtype == torch.int32
-        S = k.shape[2]
-        W = 0 if self.q is None else self.q.shape[2]
-        if self.q is not None:
-            assert self.q.is_contiguous() and self.q.dtype == k.dtype
-        P = 0 if self.page_start is None else self.page_start.numel()
-        return Traj(_ptr(k), _ptr(v), k.stride(0), k.stride(1), k.stride(2), _ptr(self.pos), S,
-                    _ptr(self.q), _ptr(self.q_pos), W, _ptr(self.page_start), _ptr(self.page_len), P)
+        i32 = _torch().int32
+        k, v, q, ps = self.k, self.v, self.q, self.page_start
+        ints = (self.pos, self.q_pos, ps, self.page_len)
+        _require_cuda(k, v, q, *ints)
+        strides, shape = k.stride(), k.shape
+        assert len(shape) == 4 and strides == v.stride() and shape == v.shape
+        assert strides[3] == 1, "head_dim must be contiguous"
+        for t in ints:
+            assert t is None or t.dtype == i32
+        if q is not None:
+            assert q.is_contiguous() and q.dtype == k.dtype
+        pos, q_pos, start, length = map(_ptr, ints)
+        return Traj(_ptr(k), _ptr(v), strides[0], strides[1], strides[2], pos, shape[2], _ptr(q), q_pos,
+                    0 if q is None else q.shape[2], start, length, 0 if ps is None else ps.numel())
 
 
 def make_shape(M, H, Hq, d, dtype, softmax_scale=0.0) -> Shape:
@@ -209,10 +211,7 @@ def _descs(trajs: Sequence[TrajTensors]):
     n = len(trajs)
     if not 1 <= n <= MAX_TRAJ:
         raise ValueError("1 <= n_traj <= 64")
-    arr = (Traj * n)()
-    for i, t in enumerate(trajs):
-        arr[i] = t.desc()
-    return arr
+    return (Traj * n)(*[t.desc() for t in trajs])
 
 
 def _mask(layer_mask, M):

@@ -43,6 +43,8 @@ from __future__ import annotations
 
 import math
 
+import numpy as np
+
 from . import commitkv as ck
 
 
@@ -78,11 +80,13 @@ class Session:
 
     # ---------------------------------------------------------------- helpers
     def _traj(self, Q=None, qpos=None) -> ck.TrajTensors:
-        torch = _torch()
-        ps = torch.tensor([p[1] for p in self.pages], dtype=torch.int32, device=self.dev)
-        pl = torch.tensor([p[2] for p in self.pages], dtype=torch.int32, device=self.dev)
+        ps, pl = self._upload(np.array([[p[1] for p in self.pages], [p[2] for p in self.pages]], np.int32))
         S = self.S
         return ck.TrajTensors(self.K[:, :, :S], self.V[:, :, :S], self.pos[:S], Q, qpos, ps, pl)
+
+    def _upload(self, rows):
+        """Rows of a host int32 array [n][P] as device tensors, in one copy."""
+        return _torch().from_numpy(rows).to(self.dev)
 
     def _workspace(self, traj):
         need = ck.commitkv_workspace_size(self.shape, [traj])
@@ -197,13 +201,13 @@ class Session:
         torch = _torch()
         s = self.shape
         S = self.S
-        none = torch.zeros(0, dtype=torch.int32, device=self.dev)
+        none = torch.empty(0, dtype=torch.int32, device=self.dev)
         tr = ck.TrajTensors(self.K[:, :, :S], self.V[:, :, :S], self.pos[:S], Q, qpos, none, none)
-        ws = self._workspace(self._traj())
-        stats = torch.zeros(s.layers, s.q_heads, Q.shape[2], s.head_dim + 4, device=self.dev)
-        R = torch.zeros(1, device=self.dev)
-        ck.commitkv_page_effects(s, [tr], [R], stats_out=[stats], workspace=ws)
-        scores = torch.zeros(max(S, 1), device=self.dev)
+        ws = self._workspace(tr)
+        # both are written in full by the calls
+        stats = torch.empty(s.layers, s.q_heads, Q.shape[2], s.head_dim + 4, device=self.dev)
+        scores = torch.empty(max(S, 1), device=self.dev)
+        ck.commitkv_page_effects(s, [tr], [scores[:0]], stats_out=[stats], workspace=ws)
         ck.commitkv_token_scores(s, [tr], [stats], [scores[:S]], workspace=ws)
         self._check()
         return scores[:S]
@@ -222,29 +226,27 @@ class Session:
         ws = self._workspace(tr)
         ids = self.page_ids()
         P, B = len(ids), self.B
-        retired = torch.tensor([1 if pid in self.retired else 0 for pid in ids], dtype=torch.uint8,
-                               device=self.dev)
         wait = set(self.measured)
         pend = [i for i, pid in enumerate(ids) if pid in wait]
-        pending = torch.tensor(pend, dtype=torch.int32, device=self.dev)
-        prio_p = torch.zeros(max(P, 1), dtype=torch.float32, device=self.dev)
-        if P:
-            prio_p[:P] = torch.tensor([self.R_pre.get(pid, 0.0) for pid in ids], dtype=torch.float32)
-        idx = torch.full((max(B, 1),), -1, dtype=torch.int32, device=self.dev)
-        n_idx = torch.zeros(1, dtype=torch.int32, device=self.dev)
+        # pending pages, priorities and retired marks in one copy
+        rows = np.zeros((3, max(P, 1)), np.int32)
+        rows[0, :len(pend)] = pend
+        rows[1, :P].view(np.float32)[:] = [self.R_pre.get(pid, 0.0) for pid in ids]
+        rows[2].view(np.uint8)[:P] = [pid in self.retired for pid in ids]
+        rows = self._upload(rows)
+        pending, prio_p, retired = rows[0, :len(pend)], rows[1].view(torch.float32), rows[2].view(torch.uint8)
+        out = torch.empty(max(B, 1) + 1, dtype=torch.int32, device=self.dev)
+        idx, n_idx = out[1:], out[:1]
         ck.commitkv_compact_in_place(self.shape, [tr], [retired], [pending], [prio_p], [fill[:self.S]], B,
                                      self.B_N, self.protect_cap, [idx], n_idx, workspace=ws)
         self._check()
-        n = int(n_idx[0])
-        I = idx[:n].cpu().tolist()
-        # page spans from the retained indices
-        new_index = {old: new for new, old in enumerate(I)}
-        pages = []
-        for pid, s, m in self.pages:
-            kept = [new_index[i] for i in range(s, s + m) if i in new_index]
-            if kept:
-                pages.append([pid, kept[0], len(kept)])
-        self.pages, self.S = pages, n
+        host = out.cpu().numpy()
+        n = int(host[0])
+        # page spans from the retained indices, which ascend: a page's kept
+        # tokens are those from its start to its end
+        spans = np.array([(s, s + m) for _, s, m in self.pages], np.int32).reshape(-1, 2)
+        spans = np.searchsorted(host[1:1 + n], spans).tolist()
+        self.pages, self.S = [[pid, a, b - a] for pid, (a, b) in zip(ids, spans) if b > a], n
         self.retired &= set(self.page_ids())
         self.decoded_since = 0
         return idx[:n]
