@@ -123,15 +123,33 @@ void fill_batch(Batch &b, const commitkv_shape *s, int n_traj, const commitkv_tr
   for (int t = 0; t < n_traj; ++t) b.t[t] = to_dev(tr[t]);
 }
 
-int chunk_len_for(int n_traj, const commitkv_traj *tr) {
+int cdiv(int a, int b) { return (a + b - 1) / b; }
+
+// ---- CUDA-core scoring path: tokens per pass-A block
+int64_t simt_units(const commitkv_shape *s, int n_layers, int n_traj, const commitkv_traj *tr, int chunk) {
+  const int g = s->q_heads / s->kv_heads;
+  int64_t units = 0;
+  for (int t = 0; t < n_traj; ++t)
+    units += (int64_t)n_layers * s->kv_heads * cdiv(g * tr[t].W, simt_rows_per_block()) * cdiv(tr[t].S, chunk);
+  return units;
+}
+
+// A call that gives few blocks takes shorter chunks, down to 128 tokens, as
+// long as they stay below this number (the fp32 Tiny workload, 18 blocks of
+// 512 tokens: pass A 161 us; 72 blocks of 128: 18 us with the merge of eight rows); larger calls at most 16
+// chunks per (layer, KV head), at least 512 tokens each.
+constexpr int64_t kSimtMaxSmallUnits = 1024;
+constexpr int kSimtMinChunk = 128;
+
+int chunk_len_for(const commitkv_shape *s, int n_layers, int n_traj, const commitkv_traj *tr) {
+  for (int c = kSimtMinChunk; c < 512; c *= 2)
+    if (simt_units(s, n_layers, n_traj, tr, c) <= kSimtMaxSmallUnits) return c;
   int smax = 0;
   for (int t = 0; t < n_traj; ++t) smax = tr[t].S > smax ? tr[t].S : smax;
   int c = (smax + 15) / 16;
   if (c < 512) c = 512;
   return (c + 63) / 64 * 64;
 }
-
-int cdiv(int a, int b) { return (a + b - 1) / b; }
 
 // ---- tensor-core scoring path (bf16)
 int tc_chunk_len(int n_traj, const commitkv_traj *tr) {
@@ -182,6 +200,18 @@ int tc_chunk_bound(int S) {
 int simt_chunk_bound(int S) {
   int c = cdiv(S, 512);
   return c < 16 ? c : 16;
+}
+
+// Partials of the CUDA-core path for these caches or smaller ones, in units of
+// a block's rows.
+size_t simt_unit_bound(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  const int g = s->q_heads / s->kv_heads;
+  size_t units = 0;
+  for (int t = 0; t < n_traj; ++t)
+    units += (size_t)s->layers * s->kv_heads * simt_chunk_bound(tr[t].S) * cdiv(g * tr[t].W, simt_rows_per_block());
+  const int64_t small = simt_units(s, s->layers, n_traj, tr, kSimtMinChunk);
+  const size_t few = (size_t)(small < kSimtMaxSmallUnits ? small : kSimtMaxSmallUnits);
+  return units > few ? units : few;
 }
 
 // The single cooperative launch of both scoring passes is opt-in
@@ -238,17 +268,13 @@ size_t tc_score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *
 }
 
 // Region sizes of each call (bytes after the 256-byte header).
-size_t score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr, int n_layers) {
-  int CL = chunk_len_for(n_traj, tr), RB = simt_rows_per_block(), d = s->head_dim;
-  int g = s->q_heads / s->kv_heads;
-  size_t units = 0, stats = 0;
-  (void)CL;
+size_t score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  int RB = simt_rows_per_block(), d = s->head_dim;
+  size_t stats = 0;
   for (int t = 0; t < n_traj; ++t) {
-    int rows = g * tr[t].W;
-    units += (size_t)n_layers * s->kv_heads * simt_chunk_bound(tr[t].S) * cdiv(rows, RB);
     stats += align_up((size_t)s->layers * s->q_heads * tr[t].W * (d + 4) * 4) + align_up((size_t)tr[t].W * 4);
   }
-  size_t scratch = align_up(units * RB * (d + 4) * 4);
+  size_t scratch = align_up(simt_unit_bound(s, n_traj, tr) * RB * (d + 4) * 4);
   const size_t tcb = tc_score_bytes(s, n_traj, tr);
   if (tcb > scratch) scratch = tcb;
   return scratch + stats;
@@ -296,7 +322,7 @@ size_t commitkv_workspace_size(const commitkv_shape *shape, int32_t n_traj,
   if (check_trajs(shape, n_traj, trajs, false) != COMMITKV_OK) return 0;
   int32_t P[kMaxTraj];
   for (int t = 0; t < n_traj; ++t) P[t] = trajs[t].P;
-  size_t need = score_bytes(shape, n_traj, trajs, shape->layers);
+  size_t need = score_bytes(shape, n_traj, trajs);
   size_t j = joint_bytes(shape, n_traj, trajs, shape->layers);
   size_t c = classify_bytes(n_traj, P);
   size_t k = compact_bytes(n_traj, trajs);
@@ -362,14 +388,23 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   memset(&L, 0, sizeof L);
   fill_batch(L.batch, shape, n_traj, trajs, layer_mask);
   int nl = L.batch.n_layers;
-  size_t need = kAlign + score_bytes(shape, n_traj, trajs, shape->layers);
+  size_t need = kAlign + score_bytes(shape, n_traj, trajs);
   if ((st = check_ws(workspace, workspace_bytes, need))) return st;
 
-  int CL = chunk_len_for(n_traj, trajs), RB = simt_rows_per_block(), PG = simt_pages_per_block();
+  int CL = chunk_len_for(shape, nl, n_traj, trajs), RB = simt_rows_per_block(), PG = simt_pages_per_block();
+  // small calls: fewer pages per block, down to one, until there is a block
+  // per SM (Tiny, 204 pages and slices: two pages per block 42 us, one 48,
+  // four 31; two layers of four heads, W = 8: 58, 57 and 78 us)
+  for (; PG > 1; PG /= 2) {
+    int64_t blocks = 0;
+    for (int t = 0; t < n_traj; ++t)
+      blocks += (int64_t)nl * shape->kv_heads * cdiv(L.batch.g * trajs[t].W, RB) * cdiv(trajs[t].P, PG);
+    if (blocks >= 152) break;
+  }
+  L.pages_per_block = PG;
   int g = L.batch.g, d = shape->head_dim;
   L.chunk_len = CL;
   char *base = static_cast<char *>(workspace) + kAlign;
-  size_t units = 0;
   for (int t = 0; t < n_traj; ++t) {
     int rows = g * trajs[t].W;
     L.nrb[t] = cdiv(rows, RB);
@@ -378,15 +413,11 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     L.unit_off_a[t + 1] = L.unit_off_a[t] + nl * shape->kv_heads * L.nchunk[t] * L.nrb[t];
     L.unit_off_b[t + 1] = L.unit_off_b[t] + nl * shape->kv_heads * L.npg[t] * L.nrb[t];
     L.row_off[t + 1] = L.row_off[t] + nl * shape->kv_heads * rows;
-    units += (size_t)nl * shape->kv_heads * L.nchunk[t] * L.nrb[t];
   }
   float *partials = reinterpret_cast<float *>(base);
   // scratch (either path's partials) first, then the stats of trajectories
   // without stats_out; the layout is computed for every layer
-  size_t full_units = 0;
-  for (int t = 0; t < n_traj; ++t)
-    full_units += (size_t)shape->layers * shape->kv_heads * simt_chunk_bound(trajs[t].S) * L.nrb[t];
-  size_t scratch = align_up(full_units * RB * (d + 4) * 4);
+  size_t scratch = align_up(simt_unit_bound(shape, n_traj, trajs) * RB * (d + 4) * 4);
   const size_t tcb = tc_score_bytes(shape, n_traj, trajs);
   if (tcb > scratch) scratch = tcb;
   char *sbase = base + scratch;

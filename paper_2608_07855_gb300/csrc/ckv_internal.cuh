@@ -118,6 +118,7 @@ struct ScoreLaunch {
   int32_t npg[kMaxTraj];             // page groups per (layer, KV head)
   int32_t row_off[kMaxTraj + 1];     // stats row offsets (selected layers only)
   int32_t chunk_len;
+  int32_t pages_per_block;
   float *stats[kMaxTraj];            // [M][Hq][W][d + 4]
   float *R[kMaxTraj];
   float *headR[kMaxTraj];

@@ -12,7 +12,16 @@
 //            r = ||U_E - S_E o|| / ((l - S_E) ||o||)  (Eq. 6 with a = e / l),
 //            max over the block's rows into R[E] and R_head[l][h][E] (Eq. 7).
 // Scores are kept in base-2 units (scale * log2 e), fp32 throughout.
+//
+// A warp takes eight probe rows together: a lane holds two tokens of the
+// 64-token tile (K read once for the eight rows, four channels at a time) and,
+// for P V, D / 32 channels.  Row by row, with scalar loads, the fp32 Tiny
+// workload (2K tokens, one layer, two heads) spent 161 us in pass A and 179 us
+// in pass B, now 18 and 42; it is bound by latency, so small calls also take
+// shorter chunks and fewer pages per block (see api.cu).  Four layers, four
+// heads of 128 channels, 5K tokens: 1,190 -> 619 and 1,739 -> 774 us.
 #include "ckv_internal.cuh"
+#include "sm103.cuh"
 
 namespace ckv {
 namespace {
@@ -59,17 +68,54 @@ __device__ __forceinline__ void load_tile_kv(const TrajDev &tr, int l, int kvh, 
       kv = to_f32(kp[off]);
       vv = to_f32(vp[off]);
     }
-    sK[i * (D + 1) + c] = kv;
+    sK[i * (D + 4) + c] = kv;
     sV[i * D + c] = vv;
   }
   for (int i = threadIdx.x; i < kTK; i += kThreads) sPos[i] = i < nt ? tr.pos[tok0 + i] : 0x7fffffff;
 }
 
-__device__ __forceinline__ float dot_smem(const float *q, const float *k, int D) {
-  float s = 0.0f;
-#pragma unroll 8
-  for (int c = 0; c < D; ++c) s = fmaf(q[c], k[c], s);
-  return s;
+// Scaled dot products of the warp's rows with tokens lane and lane + 32 of the
+// tile (base 2), even and odd channels summed apart.
+template <int D>
+__device__ __forceinline__ void tile_scores(const float *q, const float *sK, int lane, float scale_log2,
+                                            float (&s)[kRowsPerWarp][2]) {
+  using sm103::ffma2;
+  float2 a0[kRowsPerWarp], a1[kRowsPerWarp];
+#pragma unroll
+  for (int k = 0; k < kRowsPerWarp; ++k) a0[k] = a1[k] = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+  for (int c = 0; c < D; c += 4) {
+    const float4 x = *reinterpret_cast<const float4 *>(sK + lane * (D + 4) + c);
+    const float4 y = *reinterpret_cast<const float4 *>(sK + (lane + 32) * (D + 4) + c);
+#pragma unroll
+    for (int k = 0; k < kRowsPerWarp; ++k) {
+      const float4 w = *reinterpret_cast<const float4 *>(q + k * D + c);
+      a0[k] = ffma2(make_float2(w.x, w.y), make_float2(x.x, x.y), a0[k]);
+      a0[k] = ffma2(make_float2(w.z, w.w), make_float2(x.z, x.w), a0[k]);
+      a1[k] = ffma2(make_float2(w.x, w.y), make_float2(y.x, y.y), a1[k]);
+      a1[k] = ffma2(make_float2(w.z, w.w), make_float2(y.z, y.w), a1[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kRowsPerWarp; ++k) {
+    s[k][0] = (a0[k].x + a0[k].y) * scale_log2;
+    s[k][1] = (a1[k].x + a1[k].y) * scale_log2;
+  }
+}
+
+// The lane's channels of row i of sV: lane, lane + 32, ...
+template <int D>
+__device__ __forceinline__ void v_row(const float *sV, int i, int lane, float (&v)[D / 32]) {
+#pragma unroll
+  for (int j = 0; j < D / 32; ++j) v[j] = sV[i * D + lane + 32 * j];
+}
+
+// The eight rows' weights of token i ([token][row] per warp).
+__device__ __forceinline__ void p_rows(const float *pw, int i, float (&p)[kRowsPerWarp]) {
+  static_assert(kRowsPerWarp == 8, "two float4 per token");
+  const float4 a = *reinterpret_cast<const float4 *>(pw + i * kRowsPerWarp);
+  const float4 b = *reinterpret_cast<const float4 *>(pw + i * kRowsPerWarp + 4);
+  p[0] = a.x, p[1] = a.y, p[2] = a.z, p[3] = a.w, p[4] = b.x, p[5] = b.y, p[6] = b.z, p[7] = b.w;
 }
 
 // ---------------------------------------------------------------- pass A
@@ -78,10 +124,10 @@ __global__ void __launch_bounds__(kThreads) pass_a_kernel(const __grid_constant_
                                                           float *partials) {
   extern __shared__ float smem[];
   float *sQ = smem;                       // [kRB][D]
-  float *sK = sQ + kRB * D;               // [kTK][D + 1]
-  float *sV = sK + kTK * (D + 1);         // [kTK][D]
+  float *sK = sQ + kRB * D;               // [kTK][D + 4]
+  float *sV = sK + kTK * (D + 4);         // [kTK][D]
   int *sPos = reinterpret_cast<int *>(sV + kTK * D);
-  float *sP = reinterpret_cast<float *>(sPos + kTK);  // [kWarps][kTK]
+  float *sP = reinterpret_cast<float *>(sPos + kTK);  // [kWarps][kTK][kRowsPerWarp]
 
   const Batch &b = L.batch;
   int unit = blockIdx.x;
@@ -122,34 +168,54 @@ __global__ void __launch_bounds__(kThreads) pass_a_kernel(const __grid_constant_
     __syncthreads();
     load_tile_kv<T, D>(tr, l, kvh, tok0, nt, sK, sV, sPos);
     __syncthreads();
-#pragma unroll 1
+    float s[kRowsPerWarp][2];
+    tile_scores<D>(sQ + warp * kRowsPerWarp * D, sK, lane, b.scale_log2, s);
+    float *pw = sP + warp * kTK * kRowsPerWarp;
+    unsigned live = 0;  // rows that see a token of this tile
+#pragma unroll
     for (int k = 0; k < kRowsPerWarp; ++k) {
-      const float *q = sQ + (warp * kRowsPerWarp + k) * D;
       bool v0 = lane < nt && sPos[lane] <= qp[k], v1 = lane + 32 < nt && sPos[lane + 32] <= qp[k];
-      float s0 = v0 ? dot_smem(q, sK + lane * (D + 1), D) * b.scale_log2 : kNegInf;
-      float s1 = v1 ? dot_smem(q, sK + (lane + 32) * (D + 1), D) * b.scale_log2 : kNegInf;
-      float mt = warp_max(fmaxf(s0, s1));
-      if (mt == kNegInf) continue;  // nothing visible in this tile
-      float m_new = fmaxf(m_run[k], mt);
-      float alpha = exp2f(m_run[k] - m_new);
-      float p0 = v0 ? exp2f(s0 - m_new) : 0.0f;
-      float p1 = v1 ? exp2f(s1 - m_new) : 0.0f;
+      const float mt = warp_max(fmaxf(v0 ? s[k][0] : kNegInf, v1 ? s[k][1] : kNegInf));
+      const float m_new = fmaxf(m_run[k], mt);
+      live |= (mt != kNegInf ? 1u : 0u) << k;
+      // nothing visible in this tile: every weight is 0 and the sums stay
+      const float alpha = m_run[k] == m_new ? 1.0f : exp2f(m_run[k] - m_new);
+      const float p0 = v0 ? exp2f(s[k][0] - m_new) : 0.0f;
+      const float p1 = v1 ? exp2f(s[k][1] - m_new) : 0.0f;
       l_run[k] = l_run[k] * alpha + warp_sum(p0 + p1);
       n_run[k] += __popc(__ballot_sync(0xffffffffu, v0)) + __popc(__ballot_sync(0xffffffffu, v1));
       m_run[k] = m_new;
-      float *pw = sP + warp * kTK;
-      pw[lane] = p0;
-      pw[lane + 32] = p1;
-      __syncwarp();
+      pw[lane * kRowsPerWarp + k] = p0;
+      pw[(lane + 32) * kRowsPerWarp + k] = p1;
 #pragma unroll
       for (int j = 0; j < J; ++j) O[k][j] *= alpha;
-      for (int i = 0; i < nt; ++i) {
-        float p = pw[i];
-#pragma unroll
-        for (int j = 0; j < J; ++j) O[k][j] = fmaf(p, sV[i * D + lane + 32 * j], O[k][j]);
-      }
-      __syncwarp();
     }
+    __syncwarp();
+    if (live == (1u << kRowsPerWarp) - 1u) {
+#pragma unroll 2
+      for (int i = 0; i < nt; ++i) {
+        float p[kRowsPerWarp], v[J];
+        p_rows(pw, i, p);
+        v_row<D>(sV, i, lane, v);
+#pragma unroll
+        for (int k = 0; k < kRowsPerWarp; ++k)
+#pragma unroll
+          for (int j = 0; j < J; ++j) O[k][j] = fmaf(p[k], v[j], O[k][j]);
+      }
+    } else if (live) {  // a row that sees nothing here is not touched (0 times an infinite value)
+      for (int i = 0; i < nt; ++i) {
+        float p[kRowsPerWarp], v[J];
+        p_rows(pw, i, p);
+        v_row<D>(sV, i, lane, v);
+#pragma unroll
+        for (int k = 0; k < kRowsPerWarp; ++k)
+          if ((live >> k) & 1u) {
+#pragma unroll
+            for (int j = 0; j < J; ++j) O[k][j] = fmaf(p[k], v[j], O[k][j]);
+          }
+      }
+    }
+    __syncwarp();
   }
 #pragma unroll
   for (int k = 0; k < kRowsPerWarp; ++k) {
@@ -190,20 +256,25 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const __grid_constant
     return partials + ((int64_t)unit * kRB + rl) * (D + 4);
   };
   float m = kNegInf;
-  for (int c = 0; c < nch; ++c) m = fmaxf(m, part(c)[0]);
+  for (int c = lane; c < nch; c += 32) m = fmaxf(m, part(c)[0]);
+  m = warp_max(m);
   constexpr int J = D / 32;
   float o[J];
 #pragma unroll
   for (int j = 0; j < J; ++j) o[j] = 0.0f;
   float lsum = 0.0f, n = 0.0f;
+#pragma unroll 4
   for (int c = 0; c < nch; ++c) {
     const float *p = part(c);
+    const float pm = p[0];
+    float v[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) v[j] = p[4 + lane + 32 * j];
     n += p[2];
-    if (p[0] == kNegInf) continue;
-    float a = exp2f(p[0] - m);
+    const float a = pm == kNegInf ? 0.0f : exp2f(pm - m);
     lsum = fmaf(p[1], a, lsum);
 #pragma unroll
-    for (int j = 0; j < J; ++j) o[j] = fmaf(p[4 + lane + 32 * j], a, o[j]);
+    for (int j = 0; j < J; ++j) o[j] = fmaf(pm == kNegInf ? 0.0f : v[j], a, o[j]);
   }
   float inv = lsum > 0.0f ? 1.0f / lsum : 0.0f;
   int h = kvh * b.g + row / tr.W, w = row % tr.W;
@@ -219,7 +290,7 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const __grid_constant
 }
 
 // ---------------------------------------------------------------- pass B
-constexpr int kPG = 16;  // pages per block
+constexpr int kPG = 16;  // pages per block at most
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant__ ScoreLaunch L,
@@ -227,10 +298,10 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
   extern __shared__ float smem[];
   float *sQ = smem;
   float *sK = sQ + kRB * D;
-  float *sV = sK + kTK * (D + 1);
+  float *sV = sK + kTK * (D + 4);
   int *sPos = reinterpret_cast<int *>(sV + kTK * D);
   float *sP = reinterpret_cast<float *>(sPos + kTK);
-  float *sR = sP + kWarps * kTK;  // [kPG] block max per page
+  float *sR = sP + kWarps * kTK * kRowsPerWarp;  // [kPG] block max per page
 
   const Batch &b = L.batch;
   int unit = blockIdx.x;
@@ -274,9 +345,14 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
     onorm[k] = sqrtf(warp_sum(ss));
   }
 
-  int E0 = pg * kPG, E1 = min(tr.P, E0 + kPG);
+  int E0 = pg * L.pages_per_block, E1 = min(tr.P, E0 + L.pages_per_block);
   for (int e = threadIdx.x; e < kPG; e += kThreads) sR[e] = 0.0f;
   __syncthreads();
+  float *pw = sP + warp * kTK * kRowsPerWarp;
+  float S_E[kRowsPerWarp], U[kRowsPerWarp][J];
+  int n_E[kRowsPerWarp];
+  int w0 = 0, w1 = 0;  // tokens of the tile in shared memory
+  unsigned seen[kRowsPerWarp][2];
   for (int E = E0; E < E1; ++E) {
     int ps = tr.ps[E], pl = tr.pl[E];
     bool bad = pl < 0 || ps < 0 || ps > tr.S - pl || (E > 0 && ps < tr.ps[E - 1] + tr.pl[E - 1]);
@@ -284,8 +360,6 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
       if (threadIdx.x == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, E);
       continue;
     }
-    float S_E[kRowsPerWarp], U[kRowsPerWarp][J];
-    int n_E[kRowsPerWarp];
 #pragma unroll
     for (int k = 0; k < kRowsPerWarp; ++k) {
       S_E[k] = 0.0f;
@@ -293,44 +367,68 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
 #pragma unroll
       for (int j = 0; j < J; ++j) U[k][j] = 0.0f;
     }
-    for (int tok0 = ps; tok0 < ps + pl; tok0 += kTK) {
-      int nt = min(kTK, ps + pl - tok0);
-      __syncthreads();
-      load_tile_kv<T, D>(tr, l, kvh, tok0, nt, sK, sV, sPos);
-      __syncthreads();
-#pragma unroll 1
-      for (int k = 0; k < kRowsPerWarp; ++k) {
-        if (hrow[k] < 0) continue;
-        const float *q = sQ + (warp * kRowsPerWarp + k) * D;
-        bool v0 = lane < nt && sPos[lane] <= qp[k], v1 = lane + 32 < nt && sPos[lane + 32] <= qp[k];
-        float e0 = v0 ? exp2f(dot_smem(q, sK + lane * (D + 1), D) * b.scale_log2 - m2[k]) : 0.0f;
-        float e1 = v1 ? exp2f(dot_smem(q, sK + (lane + 32) * (D + 1), D) * b.scale_log2 - m2[k]) : 0.0f;
-        S_E[k] += warp_sum(e0 + e1);
-        n_E[k] += __popc(__ballot_sync(0xffffffffu, v0)) + __popc(__ballot_sync(0xffffffffu, v1));
-        float *pw = sP + warp * kTK;
-        pw[lane] = e0;
-        pw[lane + 32] = e1;
-        __syncwarp();
-        for (int i = 0; i < nt; ++i) {
-          float p = pw[i];
+    for (int tok = ps; tok < ps + pl;) {
+      if (tok < w0 || tok >= w1) {  // the next 64 tokens from here: several pages where they are short
+        w0 = tok;
+        w1 = min(tr.S, w0 + kTK);
+        const int nt = w1 - w0;
+        __syncthreads();
+        load_tile_kv<T, D>(tr, l, kvh, w0, nt, sK, sV, sPos);
+        __syncthreads();
+        float s[kRowsPerWarp][2];
+        tile_scores<D>(sQ + warp * kRowsPerWarp * D, sK, lane, b.scale_log2, s);
 #pragma unroll
-          for (int j = 0; j < J; ++j) U[k][j] = fmaf(p, sV[i * D + lane + 32 * j], U[k][j]);
+        for (int k = 0; k < kRowsPerWarp; ++k) {
+          const bool v0 = lane < nt && sPos[lane] <= qp[k], v1 = lane + 32 < nt && sPos[lane + 32] <= qp[k];
+          pw[lane * kRowsPerWarp + k] = v0 ? exp2f(s[k][0] - m2[k]) : 0.0f;
+          pw[(lane + 32) * kRowsPerWarp + k] = v1 ? exp2f(s[k][1] - m2[k]) : 0.0f;
+          seen[k][0] = __ballot_sync(0xffffffffu, v0);
+          seen[k][1] = __ballot_sync(0xffffffffu, v1);
         }
         __syncwarp();
       }
+      const int i0 = tok - w0, i1 = min(ps + pl, w1) - w0;
+      // the bits of tokens [i0, i1) of the tile
+      auto bits = [&](int base) {
+        const int a = max(i0 - base, 0), z = min(i1 - base, 32);
+        return z <= a ? 0u : (z == 32 ? 0xffffffffu : (1u << z) - 1u) & ~((1u << a) - 1u);
+      };
+      const unsigned b0 = bits(0), b1 = bits(32);
+#pragma unroll
+      for (int k = 0; k < kRowsPerWarp; ++k) n_E[k] += __popc(seen[k][0] & b0) + __popc(seen[k][1] & b1);
+#pragma unroll 2
+      for (int i = i0; i < i1; ++i) {
+        float p[kRowsPerWarp], v[J];
+        p_rows(pw, i, p);
+        v_row<D>(sV, i, lane, v);
+#pragma unroll
+        for (int k = 0; k < kRowsPerWarp; ++k) {
+          S_E[k] += p[k];
+#pragma unroll
+          for (int j = 0; j < J; ++j) U[k][j] = fmaf(p[k], v[j], U[k][j]);
+        }
+      }
+      tok = w0 + i1;
     }
+    float ss[kRowsPerWarp];
+#pragma unroll
+    for (int k = 0; k < kRowsPerWarp; ++k) {
+      ss[k] = 0.0f;
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        float dlt = fmaf(-S_E[k], o[k][j], U[k][j]);
+        ss[k] = fmaf(dlt, dlt, ss[k]);
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+      for (int k = 0; k < kRowsPerWarp; ++k) ss[k] += __shfl_xor_sync(0xffffffffu, ss[k], off);
     float rmax = 0.0f;
 #pragma unroll
     for (int k = 0; k < kRowsPerWarp; ++k) {
       if (hrow[k] < 0) continue;
-      float ss = 0.0f;
-#pragma unroll
-      for (int j = 0; j < J; ++j) {
-        float dlt = fmaf(-S_E[k], o[k][j], U[k][j]);
-        ss = fmaf(dlt, dlt, ss);
-      }
-      float num2 = warp_sum(ss);
-      float r = effect_value(n_E[k], nvis[k], S_E[k], lsum[k], num2, onorm[k]);
+      float r = effect_value(n_E[k], nvis[k], S_E[k], lsum[k], ss[k], onorm[k]);
       rmax = fmaxf(rmax, r);
       if (lane == 0 && L.headR[t])
         atomic_max_nonneg(L.headR[t] + ((int64_t)l * b.Hq + hrow[k]) * tr.P + E, r);
@@ -360,7 +458,7 @@ __global__ void __launch_bounds__(256) count_visible_kernel(const __grid_constan
 
 template <typename T, int D>
 cudaError_t launch_typed(const ScoreLaunch &L, float *partials, WsHeader *hdr, cudaStream_t s) {
-  size_t smem = (size_t)(kRB * D + kTK * (D + 1) + kTK * D) * 4 + kTK * 4 + kWarps * kTK * 4 + kPG * 4;
+  size_t smem = (size_t)(kRB * D + kTK * (D + 4) + kTK * D) * 4 + kTK * 4 + kWarps * kTK * kRowsPerWarp * 4 + kPG * 4;
   cudaError_t e;
   e = cudaFuncSetAttribute(pass_a_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
