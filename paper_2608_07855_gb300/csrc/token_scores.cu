@@ -12,13 +12,17 @@
 // kernel, one CTA of 320 threads per SM, items (trajectory, layer, KV head,
 // token chunk, 128-row tile of probe rows), the row tiles of one chunk
 // adjacent so that their K re-reads hit L2.  Per 128-token tile of K:
-//   warp 0  TMA: Q tile once per item, K tiles through a 4-stage ring
+//   warp 0  TMA: Q tile once per item (two buffers: the next item's copies
+//           start while this one's tiles are multiplied), K tiles through a ring of four stages
 //   warp 1  D[token][row] = K Q^T (tcgen05, fp32 in TMEM, two buffers)
 //   warps 2..9  two groups of four taking alternate tiles, one thread per
-//           token (TMEM lane): for every row p, 2^(s c - m_p log2 e -
-//           log2 l_p) on the rows that see the token (all of them for the
-//           tokens at or before the smallest window position), max, and one
-//           atomic max into the token's score.
+//           token (TMEM lane): the maximum over the rows p that see the token
+//           (all of them for the tokens at or before the smallest window
+//           position) of s c - m_p log2 e - log2 l_p, 2 to that power, and one
+//           atomic max into the token's score.  (An exponential per row kept
+//           the special-function unit busy for 1,024 of 2,130 cycles per
+//           tile: 36 layers of 36.9K tokens 563 us, 520 so, 496 with the second
+//           Q buffer.)
 // K rows are the MMA's M operand, so each thread reads its own token's row
 // of scores and the max over probe rows needs no cross-thread reduction.
 // CUDA-core path (fp32, head_dim 64, other layouts): one thread per token,
@@ -97,12 +101,12 @@ __device__ __forceinline__ void tma4(void *dst, const CUtensorMap *m, int x, int
 }
 
 struct Smem {
-  alignas(1024) uint8_t q[kTileBytes];
+  alignas(1024) uint8_t q[2][kTileBytes];
   alignas(1024) uint8_t k[NST][kTileBytes];
   // per epilogue warp: its own copy of the item's row terms (no cross-warp barrier)
-  float mlog[8][BR];  // row max + log2(row sum), base 2; +inf: the row sees nothing
+  alignas(16) float neg_mlog[8][BR];  // -(row max + log2(row sum)), base 2; -inf: the row sees nothing
   int qp[8][BR];      // window position of the row
-  uint64_t q_full, q_empty, k_full[NST], k_empty[NST], d_full[2], d_empty[2], drain;
+  uint64_t q_full[2], q_empty[2], k_full[NST], k_empty[NST], d_full[2], d_empty[2], drain;
   uint32_t tmem;
   int abort_flag;
 };
@@ -115,8 +119,10 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
   volatile int *abort_flag = &sm.abort_flag;
   if (threadIdx.x == 0) {
     sm.abort_flag = 0;
-    mbar_init(&sm.q_full, 1);
-    mbar_init(&sm.q_empty, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&sm.q_full[i], 1);
+      mbar_init(&sm.q_empty[i], 1);
+    }
     for (int s = 0; s < NST; ++s) {
       mbar_init(&sm.k_full[s], 1);
       mbar_init(&sm.k_empty[s], 1);
@@ -148,11 +154,12 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
         const Item a = decode(L, item);
         const TsTraj &tr = L.t[a.t];
         const tc::TcMaps &mp = L.maps[a.t];
-        if (n_local > 0 && !mbar_wait(&sm.q_empty, (n_local - 1) & 1, kWait, abort_flag)) break;
-        mbar_expect_tx(&sm.q_full, kTileBytes);
+        const int qb = n_local & 1;
+        if (n_local > 1 && !mbar_wait(&sm.q_empty[qb], ((n_local >> 1) - 1) & 1, kWait, abort_flag)) break;
+        mbar_expect_tx(&sm.q_full[qb], kTileBytes);
         const int qrow = (a.l * L.Hq + a.kvh * L.g) * tr.W + a.rt * BR;
-        tma_load_2d(sm.q, &mp.q, 0, qrow, &sm.q_full, pol);
-        tma_load_2d(sm.q + kHalf, &mp.q, 64, qrow, &sm.q_full, pol);
+        tma_load_2d(sm.q[qb], &mp.q, 0, qrow, &sm.q_full[qb], pol);
+        tma_load_2d(sm.q[qb] + kHalf, &mp.q, 64, qrow, &sm.q_full[qb], pol);
         const int t0 = a.c * kTilesPerItem * BT, t1 = min(tr.S, t0 + kTilesPerItem * BT);
         for (int tok = t0; tok < t1; tok += BT, ++g) {
           const int s = g % NST;
@@ -170,7 +177,8 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
         // let the copies already issued land before the CTA leaves
         for (uint32_t u = (n_k > NST ? n_k - NST : 0); u < n_k; ++u)
           mbar_wait_drain(&sm.k_full[u % NST], (u / NST) & 1, kWait);
-        if (n_local > 0) mbar_wait_drain(&sm.q_full, (n_local - 1) & 1, kWait);
+        for (uint32_t u = (n_local > 2 ? n_local - 2 : 0); u < n_local; ++u)
+          mbar_wait_drain(&sm.q_full[u & 1], (u >> 1) & 1, kWait);
       }
     }
   } else if (warp == 1) {
@@ -184,7 +192,8 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
         const TsTraj &tr = L.t[a.t];
         const int t0 = a.c * kTilesPerItem * BT, t1 = min(tr.S, t0 + kTilesPerItem * BT);
         const int ntile = (t1 - t0 + BT - 1) / BT;
-        if (!mbar_wait(&sm.q_full, n_local & 1, kWait, abort_flag)) break;
+        const int qb = n_local & 1;
+        if (!mbar_wait(&sm.q_full[qb], (n_local >> 1) & 1, kWait, abort_flag)) break;
         tc_fence_after();
         for (int j = 0; j < ntile; ++j, ++g) {
           const int s = g % NST, b = g & 1;
@@ -196,10 +205,10 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
           tc_fence_after();
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            mma_bf16(tm + b * BR, desc_kmajor(sm.k[s], ks), desc_kmajor(sm.q, ks), idesc, ks > 0);
+            mma_bf16(tm + b * BR, desc_kmajor(sm.k[s], ks), desc_kmajor(sm.q[qb], ks), idesc, ks > 0);
           mma_commit(&sm.d_full[b]);
           mma_commit(&sm.k_empty[s]);
-          if (j + 1 == ntile) mma_commit(&sm.q_empty);
+          if (j + 1 == ntile) mma_commit(&sm.q_empty[qb]);
         }
       }
       if (*abort_flag) {
@@ -215,7 +224,8 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
     const int hb = ew >> 2;           // this group's tiles: g & 1 == hb
     const int wq = warp & 3;          // TMEM lane quarter: warps 2..5 -> 2, 3, 0, 1; 6..9 -> 2, 3, 0, 1
     const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
-    float *mlog = sm.mlog[ew];
+    float *neg_mlog = sm.neg_mlog[ew];
+    const float2 scale2 = make_float2(L.scale_log2, L.scale_log2);
     int *qp = sm.qp[ew];
     uint32_t g = 0;
     bool ok = true;
@@ -241,7 +251,7 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
             q = tr.qpos[w];
           }
         }
-        mlog[r] = ml;
+        neg_mlog[r] = -ml;
         qp[r] = q;
         qmin = min(qmin, q);
       }
@@ -261,23 +271,33 @@ __global__ void __launch_bounds__(320, 1) token_scores_tc(const __grid_constant_
           break;
         }
         tc_fence_after();
-        float best = 0.0f;
+        // the largest weight is that of the largest exponent
+        float top = -INFINITY;
+        const bool all_seen = __all_sync(0xffffffffu, seen_by_all);
 #pragma unroll 1
         for (int c0 = 0; c0 < BR; c0 += 32) {
           float x[32];
           tmem_ld32f(tm + lane_base + b * BR + c0, x);
           tmem_wait_ld();
-          if (__all_sync(0xffffffffu, seen_by_all)) {
+          float tops[4] = {top, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-            for (int r = 0; r < 32; ++r) best = fmaxf(best, fast_exp2(fmaf(x[r], L.scale_log2, -mlog[c0 + r])));
-          } else {
-#pragma unroll
-            for (int r = 0; r < 32; ++r) {
-              const float e = fast_exp2(fmaf(x[r], L.scale_log2, -mlog[c0 + r]));
-              best = pi <= qp[c0 + r] ? fmaxf(best, e) : best;
-            }
+          for (int r = 0; r < 32; r += 4) {
+            const float4 nm = *reinterpret_cast<const float4 *>(&neg_mlog[c0 + r]);
+            const float2 a = ffma2(make_float2(x[r], x[r + 1]), scale2, make_float2(nm.x, nm.y));
+            const float2 d = ffma2(make_float2(x[r + 2], x[r + 3]), scale2, make_float2(nm.z, nm.w));
+            x[r] = a.x, x[r + 1] = a.y, x[r + 2] = d.x, x[r + 3] = d.y;
           }
+          if (!all_seen) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) x[r] = pi <= qp[c0 + r] ? x[r] : -INFINITY;
+          }
+#pragma unroll
+          for (int r = 0; r < 32; r += 8)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tops[k] = fmax3(tops[k], x[r + 2 * k], x[r + 2 * k + 1]);
+          top = fmaxf(fmax3(tops[0], tops[1], tops[2]), tops[3]);
         }
+        const float best = fast_exp2(top);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.d_empty[b]);
