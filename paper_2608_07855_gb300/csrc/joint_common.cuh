@@ -91,10 +91,19 @@ __device__ __forceinline__ int round_count(const JointLaunch &L, int t, int r) {
 
 // The round's decisions, replayed from its table: bit c set = accepted.
 __device__ __forceinline__ unsigned resolve_round(const float *tab, int kc, float tau) {
+  // every entry is read before the first decision: the reads depend on
+  // nothing, the decisions on one another
+  float R[kCombos];
+#pragma unroll
+  for (int i = 0; i < kCombos; ++i) R[i] = *(volatile const float *)(tab + i);
   unsigned acc = 0;
-  for (int c = 0; c < kc; ++c) {
-    float R = *(volatile const float *)(tab + combo(c, acc));
-    if (R <= tau) acc |= 1u << c;
+#pragma unroll
+  for (int c = 0; c < kRound; ++c) {
+    float Rc = 0.0f;
+#pragma unroll
+    for (int s = 0; s < (1 << c); ++s)
+      if (acc == (unsigned)s) Rc = R[combo(c, s)];
+    if (c < kc && Rc <= tau) acc |= 1u << c;
   }
   return acc;
 }

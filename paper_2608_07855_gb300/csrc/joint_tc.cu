@@ -74,6 +74,10 @@ struct SmemJ {
   float rc_m2[kCached][kRows], rc_l[kCached][kRows], rc_SA[kCached][kRows];
   int rc_nvis[kCached][kRows], rc_qp[kCached][kRows], rc_nA[kCached][kRows];
   int pos[kRound][kCT];
+  // the round's pages of the current group's trajectory: [0] the previous round's accepted
+  // pages (to fold), [1] the candidates; {start, length}
+  int plan_n[2];
+  int2 plan[2][kRound];
   unsigned rmax[16];
   uint64_t bar;       // Q K^T done (one issuing thread)
   uint64_t bar_pv;    // P V done (two issuing threads)
@@ -168,6 +172,43 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[kSub]) {
 // Largest member of the non-empty set T (a constant after unrolling).
 __host__ __device__ constexpr int top_bit(int T) { return T >= 8 ? 3 : T >= 4 ? 2 : T >= 2 ? 1 : 0; }
 
+// The round's plan for trajectory t (every group of it in this block uses the
+// same): called by the whole block.  Worked out by every thread for every
+// group, decision after decision, it lay on each group's chain (95 candidates
+// of 36 layers of 20K tokens: 1,199 us, 1,115 so).
+__device__ __forceinline__ void make_plan(SmemJ &s, const JointLaunch &L, WsHeader *hdr, int t, int r, int kc) {
+  __syncthreads();  // the previous plan has been read
+  const TrajDev &tr = L.batch.t[t];
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x, c = lane % kRound, set = lane / kRound;  // lanes 0..3: to fold; 4..7: candidates
+    const int kp = r > 0 ? joint::round_count(L, t, r - 1) : 0;
+    const int rr = set == 0 ? r - 1 : r, n = set == 0 ? kp : kc;
+    // page spans first: they do not depend on the decisions
+    int E = -1, ps = 0, pl = 0;
+    if (set < 2 && c < n) {
+      E = L.cand[t][rr * kRound + c];
+      if (E < 0 || E >= tr.P) {
+        record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, -4);
+      } else {
+        ps = tr.ps[E];
+        pl = tr.pl[E];
+        if (pl < 0 || ps < 0 || ps > tr.S - pl) {
+          record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, E);
+          ps = pl = 0;
+        }
+      }
+    }
+    const unsigned acc = r > 0 ? joint::resolve_round(joint::round_table(L, r - 1) + t * kCombos, kp, L.tau) : 0u;
+    if (set == 0 && c < kp && ((acc >> c) & 1u)) s.plan[0][__popc(acc & ((1u << c) - 1u))] = make_int2(ps, pl);
+    if (set == 1 && c < kc) s.plan[1][c] = make_int2(ps, pl);
+    if (lane == 0) {
+      s.plan_n[0] = __popc(acc);
+      s.plan_n[1] = kc;
+    }
+  }
+  __syncthreads();
+}
+
 // One pass over the pages list[0..n) (n <= kRound).  kScan: accumulates the
 // squared norms of the subset sums over the team's channels into ss, and
 // o's into on2 (even and odd channels apart); otherwise adds the pages' D_E into D_A in the workspace.
@@ -175,7 +216,7 @@ __host__ __device__ constexpr int top_bit(int T) { return T >= 8 ? 3 : T >= 4 ? 
 // timeout.
 template <bool kScan>
 __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeader *hdr, const Group &G,
-                                         const Row &rw, const int *list, int n, bool stage_q, uint32_t tm,
+                                         const Row &rw, const int2 *list, int n, bool stage_q, uint32_t tm,
                                          uint32_t lane_base, uint32_t &phase, uint32_t &phase_pv,
                                          float2 (&ss)[kCombos], float2 &on2,
                                          float (&Sc)[kRound], int (&nc)[kRound]) {
@@ -190,17 +231,8 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
     Sc[c] = 0.0f;
     nc[c] = 0;
     if (c < n) {
-      const int E = list[c];
-      if (E < 0 || E >= tr.P) {
-        if (tid == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, -4);
-      } else {
-        ps[c] = tr.ps[E];
-        pl[c] = tr.pl[E];
-        if (pl[c] < 0 || ps[c] < 0 || ps[c] > tr.S - pl[c]) {
-          if (tid == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, E);
-          ps[c] = pl[c] = 0;
-        }
-      }
+      ps[c] = list[c].x;
+      pl[c] = list[c].y;
       nch = max(nch, (pl[c] + kCT - 1) / kCT);
     }
   }
@@ -429,22 +461,18 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
   const int ngroups = L.group_off[b.n_traj];
   for (int r = 0; r < rounds && ok; ++r) {
     float *tab_r = joint::round_table(L, r);
+    int plan_of = -1;  // trajectory of the plan in shared memory
     for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
       const Group G = decode_group(L, grp);
       const TrajDev &tr = b.t[G.t];
       const int kc = joint::round_count(L, G.t, r);
       if (kc == 0) continue;
-      // the previous round's accepted pages, in candidate order
-      int fold[kRound], nf = 0;
-      if (r > 0) {
-        const int kp = joint::round_count(L, G.t, r - 1);
-        const unsigned acc =
-            joint::resolve_round(joint::round_table(L, r - 1) + G.t * kCombos, kp, L.tau);
-        for (int c = 0; c < kp; ++c)
-          if ((acc >> c) & 1u) fold[nf++] = L.cand[G.t][(r - 1) * kRound + c];
+      if (plan_of != G.t) {
+        make_plan(s, L, hdr, G.t, r, kc);
+        plan_of = G.t;
       }
-      int cand[kRound];
-      for (int c = 0; c < kc; ++c) cand[c] = L.cand[G.t][r * kRound + c];
+      const int nf = s.plan_n[0];
+      const int2 *fold = s.plan[0], *cand = s.plan[1];
 
       Row rw;
       const int row = G.row0 + tid % kTeam;
