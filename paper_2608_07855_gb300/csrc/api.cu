@@ -434,11 +434,10 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     sbase += align_up((size_t)trajs[t].W * 4);
   }
   L.from_stats = from_stats ? 1 : 0;
-  for (int t = 0; t < n_traj; ++t) {
-    if (trajs[t].P == 0) continue;
-    cudaError_t e = cudaMemsetAsync(R_out[t], 0, (size_t)trajs[t].P * 4, stream);
-    if (e == cudaSuccess && L.headR[t])
-      e = cudaMemsetAsync(L.headR[t], 0, (size_t)shape->layers * shape->q_heads * trajs[t].P * 4, stream);
+  for (int t = 0; t < n_traj; ++t) {  // R itself is cleared by the first kernel
+    if (trajs[t].P == 0 || !L.headR[t]) continue;
+    cudaError_t e =
+        cudaMemsetAsync(L.headR[t], 0, (size_t)shape->layers * shape->q_heads * trajs[t].P * 4, stream);
     if (e != cudaSuccess) return cuda_status(e);
   }
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
@@ -687,7 +686,7 @@ commitkv_status commitkv_joint_test(const commitkv_shape *shape, int32_t n_traj,
   }
   size_t rows_full = 0;
   for (int t = 0; t < n_traj; ++t) rows_full += (size_t)shape->layers * shape->kv_heads * g * post[t].W;
-  const size_t K = (size_t)joint_round(), tab_bytes = (size_t)3 * n_traj * joint_combos() * 4;
+  const size_t K = (size_t)joint_round();
   char *base = static_cast<char *>(workspace) + kAlign;
   L.DA = reinterpret_cast<float *>(base);
   base += align_up(rows_full * d * 4);
@@ -706,14 +705,8 @@ commitkv_status commitkv_joint_test(const commitkv_shape *shape, int32_t n_traj,
   }
   L.n_cand = n_cand;
   L.tau = tau_joint;
-  cudaError_t e = cudaMemsetAsync(L.DA, 0, rows_total * d * 4, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.SA, 0, rows_full * 8, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.roundR, 0, tab_bytes, stream);
-  for (int t = 0; t < n_traj && e == cudaSuccess; ++t)
-    if (post[t].P > 0) e = cudaMemsetAsync(accepted_out[t], 0, post[t].P, stream);
-  // the barrier counters start from a known state
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
-  if (e == cudaSuccess) e = cudaMemsetAsync(&hdr->abort, 0, 3 * sizeof(int32_t), stream);
+  cudaError_t e = launch_joint_init(L, rows_total, hdr, stream);
   if (e != cudaSuccess) return cuda_status(e);
   if (rows_total == 0 || maxP == 0) return COMMITKV_OK;
   int dev = 0, sms = 0;

@@ -166,6 +166,9 @@ struct JointLaunch {
 // Tensor-core kernel (bf16, head_dim 128, 16-byte aligned rows) when the
 // launch allows it, else the CUDA-core kernel; the row-group size follows.
 cudaError_t launch_joint(const JointLaunch &L, WsHeader *hdr, cudaStream_t stream, int sm_count);
+// Clears what a launch starts from: D_A, S_A, the round tables, the accepted
+// marks and the barrier counters.
+cudaError_t launch_joint_init(const JointLaunch &L, size_t rows, WsHeader *hdr, cudaStream_t stream);
 int joint_rows_per_group(const JointLaunch &L);
 bool joint_tc_eligible(const JointLaunch &L);
 int joint_tc_rows_per_group();

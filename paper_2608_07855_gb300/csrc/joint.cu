@@ -91,6 +91,23 @@ __device__ __forceinline__ Group decode_group(const JointLaunch &L, int grp) {
   return G;
 }
 
+// One kernel in place of a memset per array.
+__global__ void __launch_bounds__(256) joint_init_kernel(const __grid_constant__ JointLaunch L, int64_t rows,
+                                                         WsHeader *hdr) {
+  const int64_t i0 = blockIdx.x * 256 + threadIdx.x, n = (int64_t)gridDim.x * 256;
+  const int64_t da4 = rows * L.batch.d / 4, sa2 = L.rows_full;
+  for (int64_t i = i0; i < da4; i += n) reinterpret_cast<float4 *>(L.DA)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int64_t i = i0; i < sa2; i += n) reinterpret_cast<float2 *>(L.SA)[i] = make_float2(0.f, 0.f);
+  for (int64_t i = i0; i < (int64_t)3 * L.batch.n_traj * kCombos; i += n) L.roundR[i] = 0.0f;
+  for (int t = 0; t < L.batch.n_traj; ++t)
+    for (int64_t i = i0; i < L.batch.t[t].P; i += n) L.accepted[t][i] = 0;
+  if (i0 == 0) {
+    hdr->abort = 0;
+    hdr->bar_count = 0;
+    hdr->bar_gen = 0;
+  }
+}
+
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constant__ JointLaunch L,
                                                          WsHeader *hdr) {
@@ -388,6 +405,13 @@ cudaError_t launch_joint_typed(const JointLaunch &L, WsHeader *hdr, cudaStream_t
 }
 
 }  // namespace
+
+cudaError_t launch_joint_init(const JointLaunch &L, size_t rows, WsHeader *hdr, cudaStream_t stream) {
+  const int64_t work = (int64_t)rows * L.batch.d / 4;
+  const int64_t blocks = work < 256 ? 1 : work / 256 < 608 ? work / 256 : 608;
+  joint_init_kernel<<<(unsigned)blocks, 256, 0, stream>>>(L, (int64_t)rows, hdr);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_joint(const JointLaunch &L, WsHeader *hdr, cudaStream_t stream, int sm_count) {
   if (joint_tc_eligible(L)) return launch_joint_tc(L, hdr, stream, sm_count);

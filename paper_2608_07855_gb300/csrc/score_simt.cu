@@ -440,10 +440,12 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
 }
 
 // Per trajectory and window position w: the number of resident tokens with
-// pos <= qpos[w] (positions increase, so a binary search).
+// pos <= qpos[w] (positions increase, so a binary search).  Also clears R, for
+// the atomic maxima that follow.
 __global__ void __launch_bounds__(256) count_visible_kernel(const __grid_constant__ ScoreLaunch L) {
   const int t = blockIdx.x;
   const TrajDev &tr = L.batch.t[t];
+  for (int E = threadIdx.x; E < tr.P; E += blockDim.x) L.R[t][E] = 0.0f;
   for (int w = threadIdx.x; w < tr.W; w += blockDim.x) {
     const int qp = tr.qpos[w];
     int a = 0, b = tr.S;

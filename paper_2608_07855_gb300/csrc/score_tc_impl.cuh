@@ -988,6 +988,7 @@ __global__ void __launch_bounds__(256) combine_tc(const __grid_constant__ TcLaun
 //   vis_all = number of leading resident tokens visible to every probe row
 //   (positions increase, so this is a prefix); nvis_w[w] = number of resident
 //   tokens visible to window position w.
+// R is cleared, for the atomic maxima that follow.
 // For a pruned launch also where the flash pass cuts its row sums (cuts,
 // tile, piece_off: a page with slots has one piece per 128-token tile that it
 // touches), and the counters of the list passes cleared.
@@ -999,6 +1000,7 @@ __global__ void __launch_bounds__(1024) prep_kernel(const __grid_constant__ TcLa
   __shared__ unsigned long long s_w[32], s_b;
   __shared__ int s_end[32], s_bend;  // largest end of the pages seen so far
   if (threadIdx.x == 0) s_b = 0ull, s_bend = 0;
+  for (int i = threadIdx.x; i < tr.P; i += 1024) tr.R[i] = 0.0f;
   const bool prune = L.prune != 0 && tr.S > 0 && tr.W > 0;
   if (prune) {
     const int ntile = (tr.S + BT - 1) / BT;
@@ -1791,23 +1793,24 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLa
     w1[i] = any && p1 > p0 + 1 ? load(p0 + 1) : none;
     v0[i] = any && lane < n ? __half_as_ushort(vn[b + lane]) : (unsigned short)0;
   }
-  float m2[4], inv_l[4], inv_o[4];
+  // share of a row = 2^(L - ref), L the piece's log2 (P and the page's own sum
+  // differ by rounding: 0.002 and 1e-6 |max| on top); dead rows have share 0
+  float ref[4], inv_o[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const bool ok = rt * BM + 4 * lane + k < L.g * tr.W;
     const float4 a = ok ? pr.aux[(int64_t)unit * BM + 4 * lane + k] : make_float4(-INFINITY, 0.0f, 1.0f, 0.0f);
     const bool live = a.x != -INFINITY;  // the row sees something
-    m2[k] = live ? a.x - (1e-3f + 1e-6f * fabsf(a.x)) : INFINITY;
-    inv_l[k] = live ? 1.002f / a.y : 0.0f;
+    ref[k] = live ? a.x - (4e-3f + 1e-6f * fabsf(a.x)) + fast_log2(a.y) : INFINITY;
     inv_o[k] = !live ? 0.0f : a.z > 1e-15f && a.z < 1e30f ? 1.01f / a.z : INFINITY;
   }
   auto add = [&](float (&S)[4], uint2 w) {
     const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
     const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&w.y));
-    S[0] += fast_exp2(a.x - m2[0]);
-    S[1] += fast_exp2(a.y - m2[1]);
-    S[2] += fast_exp2(b.x - m2[2]);
-    S[3] += fast_exp2(b.y - m2[3]);
+    S[0] += fast_exp2(a.x - ref[0]);
+    S[1] += fast_exp2(a.y - ref[1]);
+    S[2] += fast_exp2(b.x - ref[2]);
+    S[3] += fast_exp2(b.y - ref[3]);
   };
   unsigned mine = 0;  // lane i: the bound of page i
 #pragma unroll
@@ -1817,8 +1820,9 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLa
     unsigned vb = v0[i];
     float S[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     add(S, w0[i]);
-    add(S, w1[i]);
-    if (i < np && p1 > p0) {  // pages of more than 32 tokens, or more than two tiles
+    if (i < np && p1 > p0) {
+      if (p1 > p0 + 1) add(S, w1[i]);
+      // pages of more than 32 tokens, or more than two tiles
       for (int k = lane + 32; k < n; k += 32) vb = max(vb, (unsigned)__half_as_ushort(vn[b + k]));
       for (int p = p0 + 2; p < p1; ++p) add(S, load(p));
     }
@@ -1826,11 +1830,8 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLa
     unsigned mx = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float s = S[k] * inv_l[k];
-      float r = __fdividef(s, 1.0f - s) * (1.0f + v * inv_o[k]);
-      if (m2[k] == INFINITY) r = 0.0f;
-      else if (!(s < 0.9f) || !(r >= 0.0f)) r = INFINITY;
-      mx = max(mx, __float_as_uint(r));
+      const float r = __fdividef(S[k], 1.0f - S[k]) * fmaf(v, inv_o[k], 1.0f);
+      mx = max(mx, S[k] < 0.9f ? __float_as_uint(r) & 0x7fffffffu : 0x7f800000u);  // a NaN stays above every bound
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if (lane == i) mine = mx;
