@@ -88,13 +88,17 @@ struct SmemJ {
 
 struct Group {
   int t, l, li, kvh, rows, row0;
+  // row 0 of the group in Q, the statistics and D_A: the rows of a KV head
+  // lie one after another in all three
+  const __nv_bfloat16 *q;
+  const float *st;
+  float *da;
 };
 
 // What a thread keeps of its probe row.
 struct Row {
   bool ok;          // inside the group
-  int64_t grow;     // index into D_A, S_A
-  const float *st;  // stats row: m, l, n, pad, o[D]
+  int64_t grow;     // index into S_A
   float m2, l;      // final max in base-2 units, exp-sum
   int nvis, qp;
   float SA;
@@ -122,6 +126,7 @@ __device__ __forceinline__ uint64_t desc_v(const uint8_t *tile, int h, int ks) {
 __device__ __forceinline__ uint32_t p_col(int c, int ks, int lo) {
   return kColS + kCT * c + 32 * (ks >> 1) + 8 * (ks & 1) + 16 * lo;
 }
+static_assert(kRound * kCT <= kThreads, "one thread per staged position");
 static_assert(kCT == 32, "one 32-column TMEM load covers a page chunk's scores");
 
 __device__ __forceinline__ Group decode_group(const JointLaunch &L, int grp) {
@@ -136,6 +141,10 @@ __device__ __forceinline__ Group decode_group(const JointLaunch &L, int grp) {
   G.l = b.layer_ids[G.li];
   G.rows = b.g * b.t[G.t].W;
   G.row0 = rb * kRows;
+  const int64_t row = ((int64_t)G.l * b.Hq + G.kvh * b.g) * b.t[G.t].W + G.row0;
+  G.q = static_cast<const __nv_bfloat16 *>(b.t[G.t].q) + row * D;
+  G.st = L.stats[G.t] + row * (D + 4);
+  G.da = L.DA + (L.row_off[G.t] + (int64_t)(G.li * b.H + G.kvh) * G.rows + G.row0) * D;
   return G;
 }
 
@@ -151,14 +160,30 @@ __device__ __forceinline__ bool wait_mma(SmemJ &s, uint64_t *bar, uint32_t &phas
 constexpr int kSub = 8;  // channels per epilogue step
 
 // Starts the copies of o and D_A of the team's 32 channels of half h of the
-// thread's row into that row of the half buffers.
-__device__ __forceinline__ void stage_half(SmemJ &s, const Row &rw, const float *DA, int h) {
-  if (!rw.ok) return;
-  const int i = threadIdx.x % kTeam, c0 = 32 * (threadIdx.x / kTeam);
+// warp's 32 rows into those rows of the half buffers, eight lanes to a row's
+// 128 bytes (each thread its own row took 32 lines per instruction and bound
+// the kernel).  The wait for them is followed by a __syncwarp.
+__device__ __forceinline__ void stage_half(SmemJ &s, const Group &G, int h) {
+  const int lane = threadIdx.x % 32, c0 = 32 * (threadIdx.x / kTeam) + 4 * (lane % 8);
+  const int i0 = threadIdx.x % kTeam - lane + lane / 8;
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
-    cp_async16(&s.oh[i][c0 + 4 * u], rw.st + 4 + 64 * h + c0 + 4 * u);
-    cp_async16(&s.dah[i][c0 + 4 * u], DA + rw.grow * D + 64 * h + c0 + 4 * u);
+    const int i = i0 + 4 * u;
+    if (G.row0 + i < G.rows) {
+      cp_async16(&s.oh[i][c0], G.st + i * (D + 4) + 4 + 64 * h + c0);
+      cp_async16(&s.dah[i][c0], G.da + i * D + 64 * h + c0);
+    }
+  }
+}
+// The same elements of D_A back to the workspace.
+__device__ __forceinline__ void unstage_half(const SmemJ &s, const Group &G, int h) {
+  const int lane = threadIdx.x % 32, c0 = 32 * (threadIdx.x / kTeam) + 4 * (lane % 8);
+  const int i0 = threadIdx.x % kTeam - lane + lane / 8;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = i0 + 4 * u;
+    if (G.row0 + i < G.rows)
+      *reinterpret_cast<float4 *>(G.da + i * D + 64 * h + c0) = *reinterpret_cast<const float4 *>(&s.dah[i][c0]);
   }
 }
 
@@ -212,65 +237,61 @@ __device__ __forceinline__ void make_plan(SmemJ &s, const JointLaunch &L, WsHead
 // One pass over the pages list[0..n) (n <= kRound).  kScan: accumulates the
 // squared norms of the subset sums over the team's channels into ss, and
 // o's into on2 (even and odd channels apart); otherwise adds the pages' D_E into D_A in the workspace.
-// S_E and n_E of every page are left in Sc and nc.  Returns false on a
-// timeout.
+// S_E and n_E of every page are left in Sc and nc.  The fold takes the
+// channel halves in the order 1, 0 and leaves o and the new D_A of half 0 in
+// the half buffers, where a scan with have_half finds them.  Returns false on
+// a timeout.
 template <bool kScan>
 __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeader *hdr, const Group &G,
-                                         const Row &rw, const int2 *list, int n, bool stage_q, uint32_t tm,
+                                         const Row &rw, const int2 *list, int n, bool stage_q, bool have_half, uint32_t tm,
                                          uint32_t lane_base, uint32_t &phase, uint32_t &phase_pv,
                                          float2 (&ss)[kCombos], float2 &on2,
                                          float (&Sc)[kRound], int (&nc)[kRound]) {
   const Batch &b = L.batch;
   const TrajDev &tr = b.t[G.t];
   const int tid = threadIdx.x, team = tid / kTeam, r = tid % kTeam;
-  int ps[kRound], pl[kRound];
   int nch = 1;
 #pragma unroll
   for (int c = 0; c < kRound; ++c) {
-    ps[c] = pl[c] = 0;
     Sc[c] = 0.0f;
     nc[c] = 0;
-    if (c < n) {
-      ps[c] = list[c].x;
-      pl[c] = list[c].y;
-      nch = max(nch, (pl[c] + kCT - 1) / kCT);
-    }
+    if (c < n) nch = max(nch, (list[c].y + kCT - 1) / kCT);
   }
   const __nv_bfloat16 *kp =
       static_cast<const __nv_bfloat16 *>(tr.k) + (int64_t)G.l * tr.sl + (int64_t)G.kvh * tr.sh;
   const __nv_bfloat16 *vp =
       static_cast<const __nv_bfloat16 *>(tr.v) + (int64_t)G.l * tr.sl + (int64_t)G.kvh * tr.sh;
 
-  for (int h = 0; h < 2; ++h) {
+  for (int hh = 0; hh < 2; ++hh) {
+    const int h = kScan ? hh : 1 - hh;
     for (int j = 0; j < nch; ++j) {
-      int nt[kRound];
-#pragma unroll
-      for (int c = 0; c < kRound; ++c) nt[c] = c < n ? min(kCT, max(0, pl[c] - j * kCT)) : 0;
-      if (h == 0 || nch > 1) {
+      // tokens of page c in this chunk
+      const auto ntok = [&](int c) { return min(kCT, max(0, list[c].y - j * kCT)); };
+      if (hh == 0 || nch > 1) {
         // ---- stage (the MMAs that read the buffers have completed)
         __syncthreads();
-        if (stage_q && h == 0 && j == 0) {
-          for (int e = tid; e < kRows * 16; e += kThreads) {
-            const int r = e >> 4, k16 = e & 15, row = G.row0 + r;
-            if (row < G.rows) {
-              const int hq = G.kvh * b.g + row / tr.W, w = row % tr.W;
-              const __nv_bfloat16 *src =
-                  static_cast<const __nv_bfloat16 *>(tr.q) + (((int64_t)G.l * b.Hq + hq) * tr.W + w) * D + 8 * k16;
-              cp_async16(s.q + (k16 >> 3) * kQHalf + sw128_offset(r, k16 & 7), src);
+        // 16 lanes copy a row of 256 bytes, the block 16 rows at a time
+        const int k16 = tid & 15, i0 = tid >> 4;
+        if (stage_q && hh == 0 && j == 0) {
+#pragma unroll
+          for (int i = i0; i < kRows; i += kThreads / 16)
+            if (G.row0 + i < G.rows)
+              cp_async16(s.q + (k16 >> 3) * kQHalf + sw128_offset(i, k16 & 7), G.q + i * D + 8 * k16);
+        }
+#pragma unroll 1
+        for (int c = 0; c < n; ++c) {
+          const int nt = ntok(c);
+#pragma unroll
+          for (int i = i0; i < kCT; i += kThreads / 16)
+            if (i < nt) {
+              const int64_t off = (int64_t)(list[c].x + j * kCT + i) * tr.st + 8 * k16;
+              cp_async16(s.k + (k16 >> 3) * kKHalf + sw128_offset(kCT * c + i, k16 & 7), kp + off);
+              cp_async16(s.v[c] + (k16 >> 3) * kVHalf + sw128_offset(i, k16 & 7), vp + off);
             }
-          }
         }
-        for (int e = tid; e < n * kCT * 16; e += kThreads) {
-          const int c = e / (kCT * 16), rem = e % (kCT * 16), i = rem >> 4, k16 = rem & 15;
-          if (i < nt[c]) {
-            const int64_t off = (int64_t)(ps[c] + j * kCT + i) * tr.st + 8 * k16;
-            cp_async16(s.k + (k16 >> 3) * kKHalf + sw128_offset(kCT * c + i, k16 & 7), kp + off);
-            cp_async16(s.v[c] + (k16 >> 3) * kVHalf + sw128_offset(i, k16 & 7), vp + off);
-          }
-        }
-        for (int e = tid; e < n * kCT; e += kThreads) {
-          const int c = e / kCT, i = e % kCT;
-          s.pos[c][i] = i < nt[c] ? tr.pos[ps[c] + j * kCT + i] : 0;
+        if (tid < n * kCT) {
+          const int c = tid / kCT, i = tid % kCT;
+          s.pos[c][i] = i < ntok(c) ? tr.pos[list[c].x + j * kCT + i] : 0;
         }
         cp_async_wait_all();
         fence_proxy_async();
@@ -296,13 +317,14 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
           tmem_wait_ld();
           // the chunk's visible tokens: positions increase along the page,
           // so they are a prefix, whole unless the row's position cuts it
+          const int nt = ntok(c);
           int ne = 0;
-          if (rw.ok && nt[c] > 0) {
-            if (s.pos[c][nt[c] - 1] <= rw.qp) {
-              ne = nt[c];
+          if (rw.ok && nt > 0) {
+            if (s.pos[c][nt - 1] <= rw.qp) {
+              ne = nt;
             } else {
 #pragma unroll 1
-              for (int i = 0; i < nt[c]; ++i) ne += s.pos[c][i] <= rw.qp ? 1 : 0;
+              for (int i = 0; i < nt; ++i) ne += s.pos[c][i] <= rw.qp ? 1 : 0;
             }
           }
           float se = 0.0f;
@@ -312,11 +334,9 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
             se += e;
             x[i] = e;
           }
-          if (h == 0) {
-            Sc[c] += se;
-            nc[c] += ne;
-            s.Sc[c][r] = Sc[c];
-            s.nc[c][r] = nc[c];
+          if (hh == 0) {
+            s.Sc[c][r] = j == 0 ? se : s.Sc[c][r] + se;
+            s.nc[c][r] = j == 0 ? ne : s.nc[c][r] + ne;
           }
           split_pack32(x, pk);
           tmem_st32(addr, pk);
@@ -332,7 +352,7 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
         const uint32_t idesc = idesc_bf16_f32(kRows, 64, 0, 1);
 #pragma unroll 1
         for (int c = tid / 32; c < n; c += 2) {
-          const int nks = max(1, (nt[c] + 15) / 16);
+          const int nks = max(1, (ntok(c) + 15) / 16);
 #pragma unroll 1
           for (int ks = 0; ks < nks; ++ks) {
             const uint64_t bd = desc_v(s.v[c], h, ks);
@@ -343,11 +363,12 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
         mma_commit(&s.bar_pv);
       }
       const bool last = j == nch - 1;
-      if (last) stage_half(s, rw, L.DA, h);  // in flight while the MMAs run
+      if (last && !(have_half && h == 0)) stage_half(s, G, h);  // in flight while the MMAs run
       if (!wait_mma(s, &s.bar_pv, phase_pv)) return false;
       if (last) {
-        cp_async_wait_all();  // the thread's own parts of the half buffers
-        if (h == 0) {
+        cp_async_wait_all();
+        __syncwarp();  // the warp's rows of the half buffers
+        if (hh == 0) {
 #pragma unroll
           for (int c = 0; c < kRound; ++c)
             if (c < n) {
@@ -358,7 +379,6 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
         // ---- epilogue over the team's 32 channels of half h, kSub at a time
 #pragma unroll 1
         for (int q = 4 * team; q < 4 * team + 4; ++q) {
-          const int ch0 = 64 * h + kSub * q;
           float o[kSub], da[kSub];
 #pragma unroll
           for (int u4 = 0; u4 < kSub / 4; ++u4) {
@@ -404,15 +424,17 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
             }
           }
           if constexpr (!kScan) {
-            if (rw.ok) {
-              float4 *pa = reinterpret_cast<float4 *>(L.DA + rw.grow * D + ch0);
+            float4 *pa = reinterpret_cast<float4 *>(&s.dah[r][kSub * q]);
 #pragma unroll
-              for (int u4 = 0; u4 < kSub / 4; ++u4)
-                pa[u4] = make_float4(da[4 * u4], da[4 * u4 + 1], da[4 * u4 + 2], da[4 * u4 + 3]);
-            }
+            for (int u4 = 0; u4 < kSub / 4; ++u4)
+              pa[u4] = make_float4(da[4 * u4], da[4 * u4 + 1], da[4 * u4 + 2], da[4 * u4 + 3]);
           }
         }
-        if constexpr (!kScan) __threadfence();  // D_A is read again through L2 by the scan
+        if constexpr (!kScan) {
+          __syncwarp();
+          unstage_half(s, G, h);  // read again by this warp
+          __threadfence();
+        }
       }
       // the epilogue's TMEM reads are done before the next MMAs write
       tc_fence_before();
@@ -477,9 +499,8 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
       Row rw;
       const int row = G.row0 + tid % kTeam;
       rw.ok = row < G.rows;
-      const int hq = G.kvh * b.g + (rw.ok ? row / tr.W : 0), w = rw.ok ? row % tr.W : 0;
       rw.grow = L.row_off[G.t] + (int64_t)(G.li * b.H + G.kvh) * G.rows + (rw.ok ? row : 0);
-      rw.st = L.stats[G.t] + (((int64_t)G.l * b.Hq + hq) * tr.W + w) * (D + 4);
+      const float *st = G.st + (rw.ok ? tid % kTeam : 0) * (D + 4);
       // the block's k-th group; its row data is read from global memory in
       // the first round and from the shared copy after that
       const int kslot = (grp - (int)blockIdx.x) / (int)gridDim.x, rr = tid % kTeam;
@@ -491,11 +512,11 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
         rw.SA = s.rc_SA[kslot][rr];
         rw.nA = s.rc_nA[kslot][rr];
       } else {
-        const float mn = rw.ok ? rw.st[0] : -__builtin_huge_valf();
+        const float mn = rw.ok ? st[0] : -__builtin_huge_valf();
         rw.m2 = mn == -__builtin_huge_valf() ? mn : mn * 1.4426950408889634f;
-        rw.l = rw.ok ? rw.st[1] : 0.0f;
-        rw.nvis = rw.ok ? (int)rw.st[2] : 0;
-        rw.qp = rw.ok ? tr.qpos[w] : -0x7fffffff;
+        rw.l = rw.ok ? st[1] : 0.0f;
+        rw.nvis = rw.ok ? (int)st[2] : 0;
+        rw.qp = rw.ok ? tr.qpos[row % tr.W] : -0x7fffffff;
         rw.SA = rw.ok ? L.SA[rw.grow * 2] : 0.0f;
         rw.nA = rw.ok ? (int)L.SA[rw.grow * 2 + 1] : 0;
       }
@@ -507,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
 #pragma unroll
       for (int i = 0; i < kCombos; ++i) ss2[i] = make_float2(0.0f, 0.0f);
       if (nf > 0) {
-        if (!run_pass<false>(s, L, hdr, G, rw, fold, nf, true, tm, lane_base, phase, phase_pv, ss2, on2p, Sc,
+        if (!run_pass<false>(s, L, hdr, G, rw, fold, nf, true, false, tm, lane_base, phase, phase_pv, ss2, on2p, Sc,
                              nc)) {
           ok = false;
           break;
@@ -531,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
         s.rc_SA[kslot][rr] = rw.SA;
         s.rc_nA[kslot][rr] = rw.nA;
       }
-      if (!run_pass<true>(s, L, hdr, G, rw, cand, kc, nf == 0, tm, lane_base, phase, phase_pv, ss2, on2p,
+      if (!run_pass<true>(s, L, hdr, G, rw, cand, kc, nf == 0, nf > 0, tm, lane_base, phase, phase_pv, ss2, on2p,
                           Sc, nc)) {
         ok = false;
         break;
@@ -555,23 +576,21 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
       }
       __syncthreads();
       {
-        const int T0 = tid < kTeam ? 1 : kSplit + 1, T1 = tid < kTeam ? kSplit : kCombos;
-        if (tid < kTeam) {
-#pragma unroll
-          for (int i = 0; i < kSplit; ++i) ss[i] += s.part[i][rr];
-          on2 += s.part[kCombos][rr];
-        } else {
-#pragma unroll
-          for (int i = kSplit; i < kCombos; ++i) ss[i] += s.part2[i - kSplit][rr];
-          on2 += s.part2[kCombos - kSplit][rr];
-        }
+        // The thread's subsets T0 .. T0 + 7, all values before the first
+        // reduction (one subset after another their divisions and roots lay
+        // on one chain).
+        const bool t1 = tid >= kTeam;
+        const float *other = t1 ? &s.part2[0][rr] : &s.part[0][rr];
+        const int T0 = t1 ? kSplit + 1 : 1;
+        on2 += t1 ? s.part2[kCombos - kSplit][rr] : s.part[kCombos][rr];
         // Eq. 6 on A u T for every non-empty subset T of the round's pages;
         // S and n added in candidate order
         const float onorm = sqrtf(on2);
+        float rv[kSplit];
 #pragma unroll
-        for (int T = 1; T < (1 << kRound); ++T) {
-          if (T >= (1 << kc)) break;
-          if (T < T0 || T > T1) continue;
+        for (int i = 0; i < kSplit; ++i) {
+          const int T = T0 + i;
+          const float v = (t1 ? (i < kCombos - kSplit ? ss[kSplit + i] : 0.0f) : ss[i]) + other[i * kRows];
           float S_tot = rw.SA;
           int n_tot = rw.nA;
 #pragma unroll
@@ -580,10 +599,15 @@ __global__ void __launch_bounds__(kThreads, 1) joint_tc_kernel(const __grid_cons
               S_tot += Sc[c];
               n_tot += nc[c];
             }
-          const float rv = rw.ok ? effect_value(n_tot, rw.nvis, S_tot, rw.l, ss[T - 1], onorm) : 0.0f;
-          const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(rv));
-          if (lane == 0) atomicMax(&s.rmax[T - 1], mx);
+          rv[i] = rw.ok ? effect_value(n_tot, rw.nvis, S_tot, rw.l, v, onorm) : 0.0f;
         }
+        unsigned mine = 0u;  // lane i: the warp's maximum of subset T0 + i
+#pragma unroll
+        for (int i = 0; i < kSplit; ++i) {
+          const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(rv[i]));
+          if (lane == i) mine = mx;
+        }
+        if (lane < kSplit && T0 + lane < (1 << kc)) atomicMax(&s.rmax[T0 + lane - 1], mine);
       }
       __syncthreads();
       if (tid < (1 << kc) - 1) atomic_max_nonneg(tab_r + G.t * kCombos + tid, __uint_as_float(s.rmax[tid]));
