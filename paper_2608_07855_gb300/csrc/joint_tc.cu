@@ -34,6 +34,12 @@
 // records COMMITKV_ERR_TIMEOUT, raises the abort flag that the grid barrier
 // watches, waits (bounded) for its MMAs in flight, frees its tensor memory
 // and returns.
+//
+// What bounds it: the chain of a block's two groups per round (95 candidates
+// of 36 layers of 20K tokens, 829 us: 24 rounds of two groups in 72K cycles;
+// of these the epilogue's packed FMAs 30 %, staging 15 %, the P V waits and
+// softmax 13 % each, the grid barrier with its stragglers 10 %, Eq. 6 and the
+// plan 15 %).  Neither memory (6 %) nor the tensor cores are near a limit.
 #include "joint_common.cuh"
 #include "sm103.cuh"
 
@@ -161,8 +167,8 @@ constexpr int kSub = 8;  // channels per epilogue step
 
 // Starts the copies of o and D_A of the team's 32 channels of half h of the
 // warp's 32 rows into those rows of the half buffers, eight lanes to a row's
-// 128 bytes (each thread its own row took 32 lines per instruction and bound
-// the kernel).  The wait for them is followed by a __syncwarp.
+// 128 bytes (each thread its own row: 32 lines per instruction; 1,117 us
+// for the 95 candidates below, 863 so).  The wait for them is followed by a __syncwarp.
 __device__ __forceinline__ void stage_half(SmemJ &s, const Group &G, int h) {
   const int lane = threadIdx.x % 32, c0 = 32 * (threadIdx.x / kTeam) + 4 * (lane % 8);
   const int i0 = threadIdx.x % kTeam - lane + lane / 8;
@@ -407,10 +413,12 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
             if constexpr (kScan) {
               on2 = ffma2(o2, o2, on2);
               float2 p[1 << kRound];
+              // all 15 subsets, also in a pass of fewer pages (their D_E are
+              // zero and the sums are not used): with a branch per subset the
+              // compiler could not interleave them (863 us, 829 so)
               p[0] = make_float2(da[i], da[i + 1]);
 #pragma unroll
               for (int T = 1; T < (1 << kRound); ++T) {
-                if (T >= (1 << n)) break;  // subsets of the pass's pages only
                 p[T] = ffma2(de[top_bit(T)], one2, p[T & ~(1 << top_bit(T))]);
                 ss[T - 1] = ffma2(p[T], p[T], ss[T - 1]);
               }
