@@ -23,6 +23,12 @@
 // The decisions and step values are those of the scan that takes one
 // candidate per barrier; deletion sums over disjoint pages add, which is what
 // Eq. 11's joint deletion needs.
+//
+// What bounds it at the sizes it serves: latency, a round being one chain of
+// reads, staging, dot products, reductions and a grid barrier.  2K tokens of
+// 64 fp32 channels, two KV heads: 97 us with four stagings and 30 butterfly
+// reductions per round, 47 with the round's pages staged together and the
+// subsets' sums reduced and evaluated one per lane.
 #include "joint_common.cuh"
 #include "commitkv_testing.h"
 
@@ -137,19 +143,16 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
       const int kc = joint::round_count(L, G.t, r);
       if (kc == 0) continue;
       __syncthreads();
-      for (int e = threadIdx.x; e < kRB * D; e += kThreads) {
-        int rr = e / D, c = e % D, row = G.row0 + rr;
-        float v = 0.0f;
-        if (row < G.rows) {
-          int h = G.kvh * b.g + row / tr.W, w = row % tr.W;
-          v = to_f32(static_cast<const T *>(tr.q)[(((int64_t)G.l * b.Hq + h) * tr.W + w) * D + c]);
-        }
-        sQ[rr * D + c] = v;
+      // the rows of a KV head lie one after another; a block with one group
+      // keeps its Q from round to round
+      if (r == 0 || ngroups > (int)gridDim.x) {
+        const T *q = static_cast<const T *>(tr.q) + (((int64_t)G.l * b.Hq + G.kvh * b.g) * tr.W + G.row0) * D;
+        for (int e = threadIdx.x; e < kRB * D; e += kThreads) sQ[e] = G.row0 + e / D < G.rows ? to_f32(q[e]) : 0.0f;
       }
       if (threadIdx.x < kCombos) s_rmax[threadIdx.x] = 0.0f;
       __syncthreads();
 
-      float m2[kRowsPerWarp], lsum[kRowsPerWarp], onorm[kRowsPerWarp], o[kRowsPerWarp][J], DA[kRowsPerWarp][J];
+      float m2[kRowsPerWarp], lsum[kRowsPerWarp], o[kRowsPerWarp][J], DA[kRowsPerWarp][J];
       float SA[kRowsPerWarp];
       int nA[kRowsPerWarp], nvis[kRowsPerWarp], qp[kRowsPerWarp];
       bool okr[kRowsPerWarp];
@@ -167,17 +170,74 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
         nvis[k] = okr[k] ? (int)st[2] : 0;
         qp[k] = okr[k] ? tr.qpos[w] : -0x7fffffff;
         const float *da = L.DA + grow[k] * D;
-        float ss = 0.0f;
 #pragma unroll
         for (int jj = 0; jj < J; ++jj) {
           const int ch = J * lane + jj;
           o[k][jj] = okr[k] ? st[4 + ch] : 0.0f;
-          ss = fmaf(o[k][jj], o[k][jj], ss);
           DA[k][jj] = okr[k] ? da[ch] : 0.0f;
         }
-        onorm[k] = sqrtf(warp_sum(ss));
         SA[k] = okr[k] ? L.SA[grow[k] * 2] : 0.0f;
         nA[k] = okr[k] ? (int)L.SA[grow[k] * 2 + 1] : 0;
+      }
+
+      const T *kp = static_cast<const T *>(tr.k) + (int64_t)G.l * tr.sl + (int64_t)G.kvh * tr.sh;
+      const T *vp = static_cast<const T *>(tr.v) + (int64_t)G.l * tr.sl + (int64_t)G.kvh * tr.sh;
+      constexpr int V8 = 16 / sizeof(T);  // elements per 16-byte load
+      // row i of the chunk buffers from token tok
+      const auto stage = [&](int i, int ch, int tok) {
+        float kv[V8], vv[V8];
+        const int64_t off = (int64_t)tok * tr.st + ch;
+        load16_f32<T>(kp + off, kv);
+        load16_f32<T>(vp + off, vv);
+#pragma unroll
+        for (int u = 0; u < V8; u += 4) {
+          *reinterpret_cast<float4 *>(sK + i * (D + 4) + ch + u) = make_float4(kv[u], kv[u + 1], kv[u + 2], kv[u + 3]);
+          *reinterpret_cast<float4 *>(sV + i * D + ch + u) = make_float4(vv[u], vv[u + 1], vv[u + 2], vv[u + 3]);
+        }
+      };
+      // the round's page spans, read side by side; pages that fit the chunk
+      // buffers together are staged together (one candidate after another,
+      // each with its own reads and staging, a round's latency was four such
+      // chains)
+      int ps[kRound], pl[kRound], at[kRound + 1];
+      {
+        int s0 = 0, s1 = 0;
+        if (lane < kc) {
+          const int E = L.cand[G.t][r * kRound + lane];
+          if (E < 0 || E >= tr.P) {
+            if (warp == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, -4);
+          } else {
+            s0 = tr.ps[E];
+            s1 = tr.pl[E];
+            if (s1 < 0 || s0 < 0 || s0 > tr.S - s1) {
+              if (warp == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, E);
+              s0 = s1 = 0;
+            }
+          }
+        }
+        at[0] = 0;
+#pragma unroll
+        for (int c = 0; c < kRound; ++c) {
+          ps[c] = __shfl_sync(0xffffffffu, s0, c);
+          pl[c] = __shfl_sync(0xffffffffu, s1, c);
+          at[c + 1] = min(at[c] + min(pl[c], kTK + 1), kTK + 1);
+        }
+      }
+      // (kTK: the rows that the buffers have; longer rounds keep one staging
+      // per candidate, which then also carries most of the round's time)
+      const bool together = at[kRound] <= kTK;
+      if (together) {
+        const auto token = [&](int i) {  // of row i
+          int tok = ps[0] + i;
+#pragma unroll
+          for (int c = 1; c < kRound; ++c)
+            if (i >= at[c]) tok = ps[c] + i - at[c];
+          return tok;
+        };
+        for (int e = threadIdx.x; e < at[kRound] * (D / V8); e += kThreads)
+          stage(e / (D / V8), (e % (D / V8)) * V8, token(e / (D / V8)));
+        for (int i = threadIdx.x; i < at[kRound]; i += kThreads) sPos[i] = tr.pos[token(i)];
+        __syncthreads();
       }
 
       // D_c, S_c, n_c of each candidate of the round
@@ -194,43 +254,19 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
 #pragma unroll
           for (int jj = 0; jj < J; ++jj) U[k][jj] = 0.0f;
         }
-        int ps = 0, pl = 0;
-        if (c < kc) {
-          int E = L.cand[G.t][r * kRound + c];
-          if (E < 0 || E >= tr.P) {
-            if (threadIdx.x == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, -4);
-          } else {
-            ps = tr.ps[E];
-            pl = tr.pl[E];
-            if (pl < 0 || ps < 0 || ps > tr.S - pl) {
-              if (threadIdx.x == 0) record_error(hdr, COMMITKV_ERR_DEVICE_INPUT, E);
-              pl = 0;
-              ps = 0;
-            }
+        for (int tok0 = ps[c]; tok0 < ps[c] + pl[c]; tok0 += kTK) {
+          const int nt = min(kTK, ps[c] + pl[c] - tok0);
+          // first buffer row; only the chunk's nt rows are staged: the scores
+          // of the other rows are masked out below and P V stops at nt
+          const int i0 = together ? at[c] : 0;
+          if (!together) {
+            __syncthreads();
+            for (int e = threadIdx.x; e < nt * (D / V8); e += kThreads)
+              stage(e / (D / V8), (e % (D / V8)) * V8, tok0 + e / (D / V8));
+            for (int i = threadIdx.x; i < nt; i += kThreads) sPos[i] = tr.pos[tok0 + i];
+            __syncthreads();
           }
-        }
-        const T *kp = static_cast<const T *>(tr.k) + (int64_t)G.l * tr.sl + (int64_t)G.kvh * tr.sh;
-        const T *vp = static_cast<const T *>(tr.v) + (int64_t)G.l * tr.sl + (int64_t)G.kvh * tr.sh;
-        for (int tok0 = ps; tok0 < ps + pl; tok0 += kTK) {
-          const int nt = min(kTK, ps + pl - tok0);
-          __syncthreads();
-          constexpr int V8 = 16 / sizeof(T);  // elements per 16-byte load
-          // only the chunk's nt rows: the scores of the other rows are masked
-          // out below and P V stops at nt
-          for (int e = threadIdx.x; e < nt * (D / V8); e += kThreads) {
-            const int i = e / (D / V8), ch = (e % (D / V8)) * V8;
-            float kv[V8], vv[V8];
-            const int64_t off = (int64_t)(tok0 + i) * tr.st + ch;
-            load16_f32<T>(kp + off, kv);
-            load16_f32<T>(vp + off, vv);
-#pragma unroll
-            for (int u = 0; u < V8; u += 4) {
-              *reinterpret_cast<float4 *>(sK + i * (D + 4) + ch + u) = make_float4(kv[u], kv[u + 1], kv[u + 2], kv[u + 3]);
-              *reinterpret_cast<float4 *>(sV + i * D + ch + u) = make_float4(vv[u], vv[u + 1], vv[u + 2], vv[u + 3]);
-            }
-          }
-          for (int i = threadIdx.x; i < kTK; i += kThreads) sPos[i] = i < nt ? tr.pos[tok0 + i] : 0;
-          __syncthreads();
+          const int r0 = min(i0 + lane, kTK - 1), r1 = min(i0 + lane + 32, kTK - 1);
           // scores of tokens lane and lane + 32 for the warp's rows (the four
           // dot products run side by side; each keeps its channel order)
           const float *q0 = sQ + (warp * kRowsPerWarp) * D;
@@ -241,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
           if (nt <= 32) {  // one token per lane (warp-uniform)
 #pragma unroll 2
             for (int ch = 0; ch < D; ch += 4) {
-              const float4 k0 = *reinterpret_cast<const float4 *>(sK + lane * (D + 4) + ch);
+              const float4 k0 = *reinterpret_cast<const float4 *>(sK + r0 * (D + 4) + ch);
 #pragma unroll
               for (int k = 0; k < kRowsPerWarp; ++k) {
                 const float4 qv = *reinterpret_cast<const float4 *>(q0 + k * D + ch);
@@ -254,8 +290,8 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
           } else
 #pragma unroll 2
           for (int ch = 0; ch < D; ch += 4) {
-            const float4 k0 = *reinterpret_cast<const float4 *>(sK + lane * (D + 4) + ch);
-            const float4 k1 = *reinterpret_cast<const float4 *>(sK + (lane + 32) * (D + 4) + ch);
+            const float4 k0 = *reinterpret_cast<const float4 *>(sK + r0 * (D + 4) + ch);
+            const float4 k1 = *reinterpret_cast<const float4 *>(sK + r1 * (D + 4) + ch);
 #pragma unroll
             for (int k = 0; k < kRowsPerWarp; ++k) {
               const float4 qv = *reinterpret_cast<const float4 *>(q0 + k * D + ch);
@@ -272,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
           float *pw = sP + warp * kRowsPerWarp * kTK;  // [token][row]
 #pragma unroll
           for (int k = 0; k < kRowsPerWarp; ++k) {
-            bool v0 = okr[k] && in0 && sPos[lane] <= qp[k], v1 = okr[k] && in1 && sPos[lane + 32] <= qp[k];
+            bool v0 = okr[k] && in0 && sPos[r0] <= qp[k], v1 = okr[k] && in1 && sPos[r1] <= qp[k];
             float e0 = v0 ? exp2f(s[k][0] * b.scale_log2 - m2[k]) : 0.0f;
             float e1 = v1 ? exp2f(s[k][1] * b.scale_log2 - m2[k]) : 0.0f;
             S_c[k] += warp_sum(e0 + e1);
@@ -282,10 +318,11 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
           }
           __syncwarp();
           static_assert(kRowsPerWarp == 2, "the weights of a token are read as one float2");
+#pragma unroll 4
           for (int i = 0; i < nt; ++i) {
             const float2 p = *reinterpret_cast<const float2 *>(pw + i * kRowsPerWarp);
             float v[J];
-            lds_vec<J>(sV + i * D + J * lane, v);
+            lds_vec<J>(sV + (i0 + i) * D + J * lane, v);
 #pragma unroll
             for (int jj = 0; jj < J; ++jj) {
               U[0][jj] = fmaf(p.x, v[jj], U[0][jj]);
@@ -310,41 +347,55 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
         }
       }
 
-      // Eq. 6 on A u B u {E_c} for every candidate c and subset B of the
-      // earlier ones, sums added in candidate order
+      // Eq. 6 on A u T for every non-empty subset T of the round's pages, sums
+      // added in candidate order (every subset adds its largest page last).
+      // The lanes' squared sums of the 15 subsets, and those of o, for both
+      // rows are 32 values: a transposing reduction leaves value l on lane l,
+      // the same additions as 32 butterflies with a fifth of the shuffles,
+      // and the lanes evaluate the subsets side by side.
+      {
+        static_assert(kRowsPerWarp == 2 && kCombos == 15, "one value per lane");
+        float v[32];
 #pragma unroll
-      for (int c = 0; c < kRound; ++c) {
-        if (c >= kc) break;
-#pragma unroll 1
-        for (int sb = 0; sb < (1 << c); ++sb) {
-          float rmax = 0.0f;
+        for (int i = 0; i < 32; ++i) v[i] = 0.0f;
 #pragma unroll
-          for (int k = 0; k < kRowsPerWarp; ++k) {
-            float x[J], S_tot = SA[k];
-            int n_tot = nA[k];
+        for (int k = 0; k < kRowsPerWarp; ++k)
 #pragma unroll
-            for (int jj = 0; jj < J; ++jj) x[jj] = DA[k][jj];
+          for (int jj = 0; jj < J; ++jj) {
+            float p[1 << kRound];
+            p[0] = DA[k][jj];
 #pragma unroll
-            for (int bb = 0; bb < kRound - 1; ++bb) {
-              if (bb < c && ((sb >> bb) & 1)) {
-#pragma unroll
-                for (int jj = 0; jj < J; ++jj) x[jj] += DE[bb][k][jj];
-                S_tot += SE[bb][k];
-                n_tot += nE[bb][k];
-              }
+            for (int T = 1; T < (1 << kRound); ++T) {
+              const int top = T >= 8 ? 3 : T >= 4 ? 2 : T >= 2 ? 1 : 0;
+              p[T] = p[T & ~(1 << top)] + DE[top][k][jj];
+              v[16 * k + T - 1] = fmaf(p[T], p[T], v[16 * k + T - 1]);
             }
-            float ss = 0.0f;
-#pragma unroll
-            for (int jj = 0; jj < J; ++jj) {
-              float dsum = x[jj] + DE[c][k][jj];
-              ss = fmaf(dsum, dsum, ss);
-            }
-            float num2 = warp_sum(ss);
-            float rr = effect_value(n_tot + nE[c][k], nvis[k], S_tot + SE[c][k], lsum[k], num2, onorm[k]);
-            if (okr[k]) rmax = fmaxf(rmax, rr);
+            v[16 * k + 15] = fmaf(o[k][jj], o[k][jj], v[16 * k + 15]);
           }
-          if (lane == 0) atomicMax(reinterpret_cast<int *>(&s_rmax[combo(c, sb)]), __float_as_int(rmax));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+          const bool up = (lane & off) != 0;
+#pragma unroll
+          for (int i = 0; i < off; ++i) {
+            const float keep = up ? v[i + off] : v[i], send = up ? v[i] : v[i + off];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+          }
         }
+        const bool k1 = lane >= 16;
+        const int T = (lane & 15) + 1;
+        const float onorm = sqrtf(__shfl_sync(0xffffffffu, v[0], lane | 15));
+        float S_tot = k1 ? SA[1] : SA[0];
+        int n_tot = k1 ? nA[1] : nA[0];
+#pragma unroll
+        for (int c = 0; c < kRound; ++c)
+          if ((T >> c) & 1) {
+            S_tot += k1 ? SE[c][1] : SE[c][0];
+            n_tot += k1 ? nE[c][1] : nE[c][0];
+          }
+        float rv = effect_value(n_tot, k1 ? nvis[1] : nvis[0], S_tot, k1 ? lsum[1] : lsum[0], v[0], onorm);
+        rv = (k1 ? okr[1] : okr[0]) ? fmaxf(0.0f, rv) : 0.0f;
+        rv = fmaxf(rv, __shfl_xor_sync(0xffffffffu, rv, 16));
+        if (lane < kCombos && T < (1 << kc)) atomicMax(reinterpret_cast<int *>(&s_rmax[lane]), __float_as_int(rv));
       }
       __syncthreads();
       if (threadIdx.x < kCombos && threadIdx.x < combo(kc, 0))
@@ -363,22 +414,28 @@ __global__ void __launch_bounds__(kThreads, 2) joint_kernel(const __grid_constan
       for (int k = 0; k < kRowsPerWarp; ++k) {
         int row = G.row0 + warp * kRowsPerWarp + k;
         if (row >= G.rows) continue;
-        int64_t gr = L.row_off[G.t] + (int64_t)(G.li * b.H + G.kvh) * G.rows + row;
-        float *da = L.DA + gr * D;
-        float *sa = L.SA + gr * 2;
-        for (int c = 0; c < kc; ++c) {
-          if (!((acc >> c) & 1u)) continue;
-          const float *de = L.DE + ((int64_t)c * rows_full + gr) * D;
+        const int64_t gr = L.row_off[G.t] + (int64_t)(G.li * b.H + G.kvh) * G.rows + row;
+        // every read before the first sum: one trip to L2, not one per page
+        float da[J], de[kRound][J];
+        float2 sa = *reinterpret_cast<const float2 *>(L.SA + gr * 2), se[kRound];
+        lds_vec<J>(L.DA + gr * D + J * lane, da);
 #pragma unroll
-          for (int jj = 0; jj < J; ++jj) {
-            const int ch = J * lane + jj;
-            da[ch] += de[ch];
+        for (int c = 0; c < kRound; ++c)
+          if ((acc >> c) & 1u) {
+            lds_vec<J>(L.DE + ((int64_t)c * rows_full + gr) * D + J * lane, de[c]);
+            se[c] = *reinterpret_cast<const float2 *>(L.SE + ((int64_t)c * rows_full + gr) * 2);
           }
-          if (lane == 0) {
-            sa[0] += L.SE[((int64_t)c * rows_full + gr) * 2];
-            sa[1] += L.SE[((int64_t)c * rows_full + gr) * 2 + 1];
+#pragma unroll
+        for (int c = 0; c < kRound; ++c)
+          if ((acc >> c) & 1u) {
+#pragma unroll
+            for (int jj = 0; jj < J; ++jj) da[jj] += de[c][jj];
+            sa.x += se[c].x;
+            sa.y += se[c].y;
           }
-        }
+        sts_vec<J>(L.DA + gr * D + J * lane, da);
+        __syncwarp();
+        if (lane == 0) *reinterpret_cast<float2 *>(L.SA + gr * 2) = sa;
       }
     }
     if (blockIdx.x == 0) joint::publish_round(L, r);

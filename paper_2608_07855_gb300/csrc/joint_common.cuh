@@ -122,15 +122,26 @@ __device__ __forceinline__ void publish_round(const JointLaunch &L, int r) {
   for (int t = threadIdx.x; t < b.n_traj; t += blockDim.x) {
     const int kc = round_count(L, t, r);
     const float *tab = round_table(L, r) + t * kCombos;
+    // every read before the first decision: this block is the last at the
+    // next barrier
+    float R[kCombos];
+    int E[kRound];
+#pragma unroll
+    for (int i = 0; i < kCombos; ++i) R[i] = *(volatile const float *)(tab + i);
+#pragma unroll
+    for (int c = 0; c < kRound; ++c) E[c] = c < kc ? L.cand[t][r * kRound + c] : -1;
     unsigned acc = 0;
-    for (int c = 0; c < kc; ++c) {
-      const int j = r * kRound + c;
-      const int E = L.cand[t][j];
-      const float R = *(volatile const float *)(tab + combo(c, acc));
-      if (L.stepR_out[t]) L.stepR_out[t][j] = R;
-      if (R <= L.tau) {
+#pragma unroll
+    for (int c = 0; c < kRound; ++c) {
+      if (c >= kc) break;
+      float Rc = 0.0f;
+#pragma unroll
+      for (int s = 0; s < (1 << c); ++s)
+        if (acc == (unsigned)s) Rc = R[combo(c, s)];
+      if (L.stepR_out[t]) L.stepR_out[t][r * kRound + c] = Rc;
+      if (Rc <= L.tau) {
         acc |= 1u << c;
-        if (E >= 0 && E < b.t[t].P) L.accepted[t][E] = 1;
+        if (E[c] >= 0 && E[c] < b.t[t].P) L.accepted[t][E[c]] = 1;
       }
     }
     float *next = round_table(L, r + 2) + t * kCombos;
