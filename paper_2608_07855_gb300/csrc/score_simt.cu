@@ -292,6 +292,21 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const __grid_constant
 // ---------------------------------------------------------------- pass B
 constexpr int kPG = 16;  // pages per block at most
 
+// x[k] on lane 4 k .. 4 k + 3.
+template <typename X>
+__device__ __forceinline__ X of_lane(const X (&x)[kRowsPerWarp], int lane) {
+  // halving selects (a chain of equal compares becomes an indexed access to
+  // local memory)
+  X r[kRowsPerWarp];
+#pragma unroll
+  for (int k = 0; k < kRowsPerWarp; ++k) r[k] = x[k];
+#pragma unroll
+  for (int n = kRowsPerWarp / 2, bit = 16; n > 0; n /= 2, bit /= 2)
+#pragma unroll
+    for (int k = 0; k < n; ++k) r[k] = (lane & bit) ? r[k + n] : r[k];
+  return r[0];
+}
+
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant__ ScoreLaunch L,
                                                           WsHeader *hdr) {
@@ -345,14 +360,22 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
     onorm[k] = sqrtf(warp_sum(ss));
   }
 
+  // What Eq. 6 takes of row lane / 4: the lanes evaluate the warp's rows side
+  // by side (every lane all eight, one after another, with a butterfly each,
+  // was half of a page's time: 2K tokens of 64 fp32 channels 42 us, 24 so;
+  // 5K tokens of 128 fp32 channels 773 us, 618 so).
+  static_assert(kRowsPerWarp == 8, "four lanes per row");
+  const float my_l = of_lane(lsum, lane), my_on = of_lane(onorm, lane);
+  const int my_nvis = of_lane(nvis, lane), my_h = of_lane(hrow, lane);
+
   int E0 = pg * L.pages_per_block, E1 = min(tr.P, E0 + L.pages_per_block);
   for (int e = threadIdx.x; e < kPG; e += kThreads) sR[e] = 0.0f;
   __syncthreads();
   float *pw = sP + warp * kTK * kRowsPerWarp;
   float S_E[kRowsPerWarp], U[kRowsPerWarp][J];
-  int n_E[kRowsPerWarp];
+  int n_E;  // of row lane / 4
   int w0 = 0, w1 = 0;  // tokens of the tile in shared memory
-  unsigned seen[kRowsPerWarp][2];
+  unsigned seen0 = 0u, seen1 = 0u;  // the tile's visible tokens, row lane / 4
   for (int E = E0; E < E1; ++E) {
     int ps = tr.ps[E], pl = tr.pl[E];
     bool bad = pl < 0 || ps < 0 || ps > tr.S - pl || (E > 0 && ps < tr.ps[E - 1] + tr.pl[E - 1]);
@@ -363,10 +386,10 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
 #pragma unroll
     for (int k = 0; k < kRowsPerWarp; ++k) {
       S_E[k] = 0.0f;
-      n_E[k] = 0;
 #pragma unroll
       for (int j = 0; j < J; ++j) U[k][j] = 0.0f;
     }
+    n_E = 0;
     for (int tok = ps; tok < ps + pl;) {
       if (tok < w0 || tok >= w1) {  // the next 64 tokens from here: several pages where they are short
         w0 = tok;
@@ -376,15 +399,18 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
         load_tile_kv<T, D>(tr, l, kvh, w0, nt, sK, sV, sPos);
         __syncthreads();
         float s[kRowsPerWarp][2];
+        unsigned seen[2][kRowsPerWarp];
         tile_scores<D>(sQ + warp * kRowsPerWarp * D, sK, lane, b.scale_log2, s);
 #pragma unroll
         for (int k = 0; k < kRowsPerWarp; ++k) {
           const bool v0 = lane < nt && sPos[lane] <= qp[k], v1 = lane + 32 < nt && sPos[lane + 32] <= qp[k];
           pw[lane * kRowsPerWarp + k] = v0 ? exp2f(s[k][0] - m2[k]) : 0.0f;
           pw[(lane + 32) * kRowsPerWarp + k] = v1 ? exp2f(s[k][1] - m2[k]) : 0.0f;
-          seen[k][0] = __ballot_sync(0xffffffffu, v0);
-          seen[k][1] = __ballot_sync(0xffffffffu, v1);
+          seen[0][k] = __ballot_sync(0xffffffffu, v0);
+          seen[1][k] = __ballot_sync(0xffffffffu, v1);
         }
+        seen0 = of_lane(seen[0], lane);
+        seen1 = of_lane(seen[1], lane);
         __syncwarp();
       }
       const int i0 = tok - w0, i1 = min(ps + pl, w1) - w0;
@@ -393,9 +419,7 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
         const int a = max(i0 - base, 0), z = min(i1 - base, 32);
         return z <= a ? 0u : (z == 32 ? 0xffffffffu : (1u << z) - 1u) & ~((1u << a) - 1u);
       };
-      const unsigned b0 = bits(0), b1 = bits(32);
-#pragma unroll
-      for (int k = 0; k < kRowsPerWarp; ++k) n_E[k] += __popc(seen[k][0] & b0) + __popc(seen[k][1] & b1);
+      n_E += __popc(seen0 & bits(0)) + __popc(seen1 & bits(32));
 #pragma unroll 2
       for (int i = i0; i < i1; ++i) {
         float p[kRowsPerWarp], v[J];
@@ -420,20 +444,28 @@ __global__ void __launch_bounds__(kThreads) pass_b_kernel(const __grid_constant_
         ss[k] = fmaf(dlt, dlt, ss[k]);
       }
     }
+    // row lane / 4 on each lane: the butterfly's additions, each row's in an
+    // eighth of the lanes from the third on
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
+    for (int off = 16, n = kRowsPerWarp / 2; off > 0; off >>= 1, n /= 2) {
+      if (n > 0) {
+        const bool up = (lane & off) != 0;
 #pragma unroll
-      for (int k = 0; k < kRowsPerWarp; ++k) ss[k] += __shfl_xor_sync(0xffffffffu, ss[k], off);
-    float rmax = 0.0f;
-#pragma unroll
-    for (int k = 0; k < kRowsPerWarp; ++k) {
-      if (hrow[k] < 0) continue;
-      float r = effect_value(n_E[k], nvis[k], S_E[k], lsum[k], ss[k], onorm[k]);
-      rmax = fmaxf(rmax, r);
-      if (lane == 0 && L.headR[t])
-        atomic_max_nonneg(L.headR[t] + ((int64_t)l * b.Hq + hrow[k]) * tr.P + E, r);
+        for (int k = 0; k < n; ++k) {
+          const float keep = up ? ss[k + n] : ss[k], send = up ? ss[k] : ss[k + n];
+          ss[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+      } else {
+        ss[0] += __shfl_xor_sync(0xffffffffu, ss[0], off);
+      }
     }
-    if (lane == 0) atomicMax(reinterpret_cast<int *>(sR + (E - E0)), __float_as_int(rmax));
+    float r = 0.0f;
+    if (my_h >= 0) {
+      r = effect_value(n_E, my_nvis, of_lane(S_E, lane), my_l, ss[0], my_on);
+      if (lane % 4 == 0 && L.headR[t]) atomic_max_nonneg(L.headR[t] + ((int64_t)l * b.Hq + my_h) * tr.P + E, r);
+    }
+    const unsigned rmax = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(0.0f, r)));
+    if (lane == 0) atomicMax(reinterpret_cast<int *>(sR + (E - E0)), (int)rmax);
   }
   __syncthreads();
   for (int E = E0 + threadIdx.x; E < E1; E += kThreads) atomic_max_nonneg(L.R[t] + E, sR[E - E0]);
