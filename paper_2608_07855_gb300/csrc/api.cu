@@ -393,8 +393,9 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
 
   int CL = chunk_len_for(shape, nl, n_traj, trajs), RB = simt_rows_per_block(), PG = simt_pages_per_block();
   // small calls: fewer pages per block, down to one, until there is a block
-  // per SM (Tiny, 204 pages and slices: two pages per block 42 us, one 48,
-  // four 31; two layers of four heads, W = 8: 58, 57 and 78 us)
+  // per SM (half as many blocks, this line, twice as many: 2K tokens of one
+  // layer and two heads 24, 24 and 30 us; two layers of four heads, 1.5K
+  // tokens, W = 8: 53, 41 and 27 us)
   for (; PG > 1; PG /= 2) {
     int64_t blocks = 0;
     for (int t = 0; t < n_traj; ++t)

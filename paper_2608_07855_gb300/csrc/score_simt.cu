@@ -17,9 +17,9 @@
 // 64-token tile (K read once for the eight rows, four channels at a time) and,
 // for P V, D / 32 channels.  Row by row, with scalar loads, the fp32 Tiny
 // workload (2K tokens, one layer, two heads) spent 161 us in pass A and 179 us
-// in pass B, now 18 and 42; it is bound by latency, so small calls also take
+// in pass B, now 18 and 24; it is bound by latency, so small calls also take
 // shorter chunks and fewer pages per block (see api.cu).  Four layers, four
-// heads of 128 channels, 5K tokens: 1,190 -> 619 and 1,739 -> 774 us.
+// heads of 128 channels, 5K tokens: 1,190 -> 619 and 1,739 -> 619 us.
 #include "ckv_internal.cuh"
 #include "sm103.cuh"
 

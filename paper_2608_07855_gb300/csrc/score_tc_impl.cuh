@@ -16,9 +16,9 @@
 //            pages of a unit that can raise R, first those of the unit with
 //            the largest bound, then those whose bound is above the effects
 //            found.  On 36 layers of 16K + 2K tokens (pages of 32): page pass
-//            1,495 us, instead bounds 61, lists 18, page pass over the rest
-//            250, and pass A 884 -> 1,099 us for the sums; 32K + 4K: scoring
-//            4.26 -> 2.6 ms.
+//            1,495 us, instead bounds 57, lists 13, page pass over the rest
+//            245, and pass A 900 -> 1,070 us for the sums; 32K + 4K: scoring
+//            4.26 -> 2.55 ms.
 //   pass B   persistent, over tiles of 8 slots: every page is loaded as
 //            16-row TMA boxes into slots of its own, so one page's columns
 //            never share a 16-wide MMA k-block with another page.
