@@ -36,7 +36,7 @@
 // and returns.
 //
 // What bounds it: the chain of a block's two groups per round (95 candidates
-// of 36 layers of 20K tokens, 829 us: 24 rounds of two groups in 72K cycles;
+// of 36 layers of 20K tokens, 802 us: 24 rounds of two groups in 69K cycles;
 // of these the epilogue's packed FMAs 30 %, staging 15 %, the P V waits and
 // softmax 13 % each, the grid barrier with its stragglers 10 %, Eq. 6 and the
 // plan 15 %).  Neither memory (6 %) nor the tensor cores are near a limit.
@@ -440,8 +440,11 @@ __device__ __forceinline__ bool run_pass(SmemJ &s, const JointLaunch &L, WsHeade
         }
         if constexpr (!kScan) {
           __syncwarp();
-          unstage_half(s, G, h);  // read again by this warp
-          __threadfence();
+          unstage_half(s, G, h);
+          // read again by this block alone (the group stays with it): no
+          // fence beyond it, whose wait for the writes lay on every fold (95
+          // candidates of 36 layers of 20K tokens: 826 us, 802 so)
+          __threadfence_block();
         }
       }
       // the epilogue's TMEM reads are done before the next MMAs write
