@@ -442,7 +442,13 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     if (e != cudaSuccess) return cuda_status(e);
   }
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
-  if (!tc_eligible(shape, n_traj, trajs)) return cuda_status(launch_score_simt(L, partials, hdr, stream));
+  // 64 channels from given statistics: on the CUDA cores.  The tensor cores'
+  // accumulation truncates U_E; with the flash pass's own o, built the same
+  // way, that cancels in U_E - S_E o (effects off by 1e-6, on the CUDA cores
+  // 5e-6), with exact statistics it does not (8e-6 to 2e-5 against 2e-6 to
+  // 5e-6, 16 layers of 2.6K to 11K tokens).
+  if (!tc_eligible(shape, n_traj, trajs) || (from_stats && d == 64))
+    return cuda_status(launch_score_simt(L, partials, hdr, stream));
   // tensor-core path: trajectories in launches of up to tc::kMaxTc
   static thread_local tc::TcLaunch T;
   int dev = 0, sms = 0;
