@@ -22,7 +22,8 @@ constexpr int kMaxPending = 2048;
 // Blocks per trajectory (one cluster): one up to kOneBlock tokens, else eight.
 // One block's dozen sweeps over 36.9K tokens took 62 us, most of it waiting
 // for its own loads and for histogram additions to the same bin; eight take
-// 33 us.  At 2,320 tokens one takes 12 us, eight 21.
+// 33 us.  At 2,400 tokens one takes 11 us, eight 15; at 7,500 17 to 20 and
+// 17 to 18, at 10,000 24 to 28 and 18 to 20.
 constexpr int kCluster = 8;
 constexpr int kOneBlock = 8192;
 constexpr int kKeys = 8;   // tokens a thread keeps in registers; longer shares are read from memory every time
