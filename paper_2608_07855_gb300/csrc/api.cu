@@ -442,11 +442,13 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     if (e != cudaSuccess) return cuda_status(e);
   }
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
-  // 64 channels from given statistics: on the CUDA cores.  The tensor cores'
-  // accumulation truncates U_E; with the flash pass's own o, built the same
-  // way, that cancels in U_E - S_E o (effects off by 1e-6, on the CUDA cores
-  // 5e-6), with exact statistics it does not (8e-6 to 2e-5 against 2e-6 to
-  // 5e-6, 16 layers of 2.6K to 11K tokens).
+  // 64 channels from given statistics: on the CUDA cores.  The rounding of the
+  // scores enters l - S_E and U_E - S_E o and cancels where the statistics
+  // were summed in the same order: those that an engine's fp32 sums give match the
+  // CUDA cores' chains (errors of 2e-6 to 5e-6, on the tensor cores 8e-6 to
+  // 2e-5; 12 to 16 layers of 2.6K to 11K tokens).  The library's own, from the
+  // tensor cores, match those instead: fed back here they are off by 8e-6 to
+  // 4e-5, where the call that made them is off by 1e-6.
   if (!tc_eligible(shape, n_traj, trajs) || (from_stats && d == 64))
     return cuda_status(launch_score_simt(L, partials, hdr, stream));
   // tensor-core path: trajectories in launches of up to tc::kMaxTc

@@ -55,7 +55,7 @@ def test_effects_and_stats_of_64_channel_heads(kw):
     assert np.all(np.abs(st[:, 0] - m) <= 1e-5 * np.abs(m) + 1e-6)
     assert np.all(np.abs(st[:, 1] - l) <= 1e-5 * l)
     assert np.all(np.linalg.norm(st[:, 4:] - o, axis=1) <= 1e-5 * np.linalg.norm(o, axis=1))
-    # the page pass alone, from the exact statistics: 2e-5 would be the tensor cores' truncation
+    # the page pass alone, from the exact statistics
     exact = np.concatenate([np.stack([m, l, n], 1), np.zeros((len(m), 1)), o], 1).astype(np.float32)
     R2 = torch.zeros_like(Rp)
     ck.commitkv_page_effects_from_stats(buf.shape, [dev.post()], [torch.from_numpy(exact).cuda().view_as(buf.stats[0])], [R2],
