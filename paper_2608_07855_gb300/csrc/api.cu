@@ -383,6 +383,40 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     if (stats_in && trajs[t].P > 0 && trajs[t].W > 0 && !stats_in[t]) return COMMITKV_ERR_INVALID_ARG;
   }
   const bool from_stats = stats_in != nullptr;
+  int n_stats = 0;  // trajectories whose row statistics the caller wants
+  for (int t = 0; stats_out && t < n_traj; ++t) n_stats += stats_out[t] != nullptr;
+  // 64 channels, statistics in or out: on the CUDA cores.  The rounding of the
+  // scores enters l - S_E and U_E - S_E o and cancels where statistics and
+  // scores are summed in the same order.  What takes statistics of this width
+  // (the single-read call, the joint test, the token scores) runs on the CUDA
+  // cores, and so do, in effect, an engine's fp32 sums: with the tensor cores'
+  // scores on one side only, effects from statistics were off by 8e-6 to 4e-5
+  // (2e-6 to 1e-5 so), joint steps by 9e-7 (1e-7), token scores by 2e-6 (5e-7).
+  // Effects alone are the more exact ones on the tensor cores (1e-6 against
+  // 5e-6) and take 245 us against 3.7 ms (16 layers of 8K tokens), so a call
+  // with both kinds of trajectories is split.
+  const bool simt64 = shape->head_dim == 64 && shape->dtype == COMMITKV_BF16 && (from_stats || n_stats > 0);
+  if (simt64 && !from_stats && n_stats < n_traj) {
+    const size_t all = kAlign + score_bytes(shape, n_traj, trajs);
+    if ((st = check_ws(workspace, workspace_bytes, all))) return st;
+    for (int with = 0; with < 2; ++with) {
+      commitkv_traj tr[COMMITKV_MAX_TRAJ];
+      float *R[COMMITKV_MAX_TRAJ], *hR[COMMITKV_MAX_TRAJ], *so[COMMITKV_MAX_TRAJ];
+      int n = 0;
+      for (int t = 0; t < n_traj; ++t) {
+        if ((stats_out[t] != nullptr) != (with == 1)) continue;
+        tr[n] = trajs[t];
+        R[n] = R_out[t];
+        hR[n] = head_R_out ? head_R_out[t] : nullptr;
+        so[n++] = stats_out[t];
+      }
+      // one after the other on the stream, in the same workspace
+      st = page_effects_impl(shape, n, tr, layer_mask, nullptr, R, head_R_out ? hR : nullptr, with ? so : nullptr,
+                             workspace, workspace_bytes, stream);
+      if (st) return st;
+    }
+    return COMMITKV_OK;
+  }
 
   static thread_local ScoreLaunch L;  // large: keep off the stack
   memset(&L, 0, sizeof L);
@@ -442,14 +476,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     if (e != cudaSuccess) return cuda_status(e);
   }
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
-  // 64 channels from given statistics: on the CUDA cores.  The rounding of the
-  // scores enters l - S_E and U_E - S_E o and cancels where the statistics
-  // were summed in the same order: those that an engine's fp32 sums give match the
-  // CUDA cores' chains (errors of 2e-6 to 5e-6, on the tensor cores 8e-6 to
-  // 2e-5; 12 to 16 layers of 2.6K to 11K tokens).  The library's own, from the
-  // tensor cores, match those instead: fed back here they are off by 8e-6 to
-  // 4e-5, where the call that made them is off by 1e-6.
-  if (!tc_eligible(shape, n_traj, trajs) || (from_stats && d == 64))
+  if (!tc_eligible(shape, n_traj, trajs) || simt64)
     return cuda_status(launch_score_simt(L, partials, hdr, stream));
   // tensor-core path: trajectories in launches of up to tc::kMaxTc
   static thread_local tc::TcLaunch T;

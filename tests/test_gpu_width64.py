@@ -30,7 +30,12 @@ def test_effects_and_stats_of_64_channel_heads(kw):
     Rp = torch.zeros(dev.P_post, device="cuda")
     ck.commitkv_page_effects(buf.shape, [dev.post()], [Rp], head_R_out=head, workspace=buf.ws)
     assert buf.status() == ck.COMMITKV_OK
-    assert torch.equal(Rp, buf.R_post[0])
+    # the same call without maxima per head, in one batch with the pre-commit cache, which
+    # both take the tensor cores; with statistics the post-commit cache took the CUDA cores
+    Rq = [torch.zeros(tr.P_pre, device="cuda"), torch.zeros(dev.P_post, device="cuda")]
+    ck.commitkv_page_effects(buf.shape, [dev.pre(), dev.post()], Rq, workspace=buf.ws)
+    assert buf.status() == ck.COMMITKV_OK
+    assert torch.equal(Rq[1], Rp) and torch.equal(Rq[0], buf.R_pre[0][:tr.P_pre])
 
     def f64(a):
         return synth.values_f64(a, "bf16")
@@ -39,7 +44,7 @@ def test_effects_and_stats_of_64_channel_heads(kw):
     pre = oracle.Problem(f64(tr.K)[:, :, :L], f64(tr.V)[:, :, :L], tr.pos[:L], f64(tr.Q_pre), tr.qpos_pre,
                          tr.page_start[:tr.P_pre], tr.page_len[:tr.P_pre])
     post = oracle.Problem(f64(tr.K), f64(tr.V), tr.pos, f64(tr.Q_post), tr.qpos_post, tr.page_start, tr.page_len)
-    for got, prob, per_head in ((buf.R_pre[0][:tr.P_pre], pre, None), (buf.R_post[0], post, head[0])):
+    for got, prob, per_head in ((Rq[0], pre, None), (Rp, post, head[0]), (buf.R_post[0], post, None)):
         want = oracle.page_effects(prob, "closed")
         for g, w in ((got, want[0]), (per_head, want[1])):
             if g is None:
@@ -66,3 +71,7 @@ def test_effects_and_stats_of_64_channel_heads(kw):
     g = R2.cpu().numpy().astype(np.float64)
     assert np.array_equal(np.isfinite(g), np.isfinite(w))
     assert np.linalg.norm(g[fin] - w[fin]) <= 1e-5 * np.linalg.norm(w[fin])
+    # from the call's own statistics: the effects of that call
+    ck.commitkv_page_effects_from_stats(buf.shape, [dev.post()], [buf.stats[0]], [R2], workspace=buf.ws)
+    assert buf.status() == ck.COMMITKV_OK
+    assert torch.equal(R2, buf.R_post[0])
