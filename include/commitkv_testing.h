@@ -27,6 +27,15 @@ extern "C" {
 commitkv_status commitkv_test_barrier_timeout(void *workspace, size_t workspace_bytes,
                                               int32_t blocks, cudaStream_t stream);
 
+/*
+ * What the last scoring launch on this workspace left to its page passes:
+ * pages_out[0] and pages_out[1] (host) receive the (row tile, page) pairs
+ * that the two list passes of the pruned page pass scored, both 0 where the
+ * full page pass ran.  Waits for the stream.
+ */
+commitkv_status commitkv_test_pruned_pages(const void *workspace, size_t workspace_bytes, uint64_t *pages_out,
+                                           cudaStream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

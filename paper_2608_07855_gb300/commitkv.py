@@ -98,11 +98,12 @@ def load_library(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.commitkv_compact_noalloc.argtypes = [P(Shape), i32, P(Traj), vp, vp, vp, vp, vp, i32, i32,
                                              i32, vp, vp, vp, vp, vp, vp, vp]
     lib.commitkv_test_barrier_timeout.argtypes = [vp, sz, i32, vp]
+    lib.commitkv_test_pruned_pages.argtypes = [vp, sz, vp, vp]
     lib.commitkv_token_scores.argtypes = [P(Shape), i32, P(Traj), vp, vp, vp, vp, sz, vp]
     for f in ("commitkv_workspace_init", "commitkv_workspace_status", "commitkv_page_effects",
               "commitkv_page_effects_from_stats", "commitkv_classify", "commitkv_classify_variant",
               "commitkv_joint_test", "commitkv_compact", "commitkv_compact_in_place", "commitkv_compact_noalloc",
-              "commitkv_test_barrier_timeout", "commitkv_token_scores"):
+              "commitkv_test_barrier_timeout", "commitkv_test_pruned_pages", "commitkv_token_scores"):
         getattr(lib, f).restype = ctypes.c_int
     _lib = lib
     return lib
@@ -258,6 +259,15 @@ def commitkv_test_barrier_timeout(ws, blocks=2, stream=None):
     _check(load_library().commitkv_test_barrier_timeout(_ptr(ws), ws.numel(), int(blocks),
                                                         _stream(stream)),
            "commitkv_test_barrier_timeout")
+
+
+def commitkv_test_pruned_pages(ws, stream=None):
+    """(row tile, page) pairs that the two list passes of the last scoring
+    launch scored; (0, 0) where the full page pass ran."""
+    out = (ctypes.c_uint64 * 2)()
+    _check(load_library().commitkv_test_pruned_pages(_ptr(ws), ws.numel(), out, _stream(stream)),
+           "commitkv_test_pruned_pages")
+    return out[0], out[1]
 
 
 def commitkv_page_effects(shape: Shape, trajs, R_out, head_R_out=None, stats_out=None,

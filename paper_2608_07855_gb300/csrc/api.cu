@@ -260,7 +260,7 @@ size_t tc_score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *
     slots += align_up((size_t)(tr[t].P + 1) * 4) + align_up((size_t)c.nbitem * 32) + kAlign +
              align_up(((size_t)cdiv(tr[t].S, 16) + tr[t].P) * 16);
     slots += tc::prune_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt) +
-             align_up(tc::prune_item_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt)) + kAlign;
+             align_up(tc::prune_item_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt));
     slices += (size_t)s->layers * s->kv_heads;
   }
   return align_up(tc_partial_slots(s, n_traj, tr) * tc::kPartsPerItem * tc::kRowsPerTile * (s->head_dim + 4) * 4) +
@@ -351,6 +351,18 @@ commitkv_status commitkv_workspace_status(const void *workspace, size_t workspac
     if (e != cudaSuccess) return cuda_status(e);
   }
   return (commitkv_status)h.status;
+}
+
+commitkv_status commitkv_test_pruned_pages(const void *workspace, size_t workspace_bytes, uint64_t *pages_out,
+                                           cudaStream_t stream) {
+  if (!workspace || workspace_bytes < kAlign || ((uintptr_t)workspace % kAlign)) return COMMITKV_ERR_WORKSPACE;
+  if (!pages_out) return COMMITKV_ERR_INVALID_ARG;
+  WsHeader h;
+  cudaError_t e = cudaMemcpyAsync(&h, workspace, sizeof h, cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (e != cudaSuccess) return cuda_status(e);
+  for (int i = 0; i < 2; ++i) pages_out[i] = h.list_work[i] >> 32;
+  return COMMITKV_OK;
 }
 
 const char *commitkv_status_string(commitkv_status s) {
@@ -539,11 +551,8 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       slot_base += align_up(((size_t)cdiv(x.S, 16) + x.P) * 16);
       {
         const int slices = shape->layers * shape->kv_heads;
-        if (T.prune) {
-          if (!T.n_list_items) T.n_list_items = reinterpret_cast<int *>(slot_base);
-          tc::prune_layout(tt.pr, slot_base + kAlign, x.S, x.P, slices, c.nrt);
-        }
-        slot_base += kAlign + tc::prune_bytes(x.S, x.P, slices, c.nrt);
+        if (T.prune) tc::prune_layout(tt.pr, slot_base, x.S, x.P, slices, c.nrt);
+        slot_base += tc::prune_bytes(x.S, x.P, slices, c.nrt);
       }
       tt.stats = L.stats[t];
       tt.nvis_w = L.nvis_w[t];

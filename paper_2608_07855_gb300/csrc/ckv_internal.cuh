@@ -39,7 +39,10 @@ struct WsHeader {
   uint32_t bar_count;       // grid barrier arrivals
   uint32_t bar_gen;         // grid barrier generation
   int32_t err_info[4];      // where the first error was seen (debug)
-  uint32_t pad[56];
+  // Pruned page pass of the last scoring launch: per list pass {pages taken
+  // << 32 | work items}; 0 where the full pass ran.
+  unsigned long long list_work[2];
+  uint32_t pad[52];
 };
 static_assert(sizeof(WsHeader) == 256, "workspace header is 256 bytes");
 

@@ -87,7 +87,6 @@ struct TcLaunch {
   int bound_off[kMaxTc + 1];  // blocks of bound_kernel: prefix per trajectory
   int seed_off[kMaxTc + 1];   // blocks of seed_kernel
   int4 *list_items;           // workspace: {unit, first entry of its list, entries, pages} of every work item
-  int *n_list_items;          // workspace [2]: items of the two list passes
   uint8_t layer_ids[kMaxLayers];
 };
 

@@ -1007,7 +1007,7 @@ __global__ void __launch_bounds__(1024) prep_kernel(const __grid_constant__ TcLa
     for (int i = threadIdx.x; i < 4 * ntile; i += 1024) tr.pr.cuts[i] = make_uint2(0u, 0u);
     for (int i = threadIdx.x; i < ntile; i += 1024) tr.pr.tile[i] = make_int2(0x7fffffff, 0);
   }
-  if (L.prune && blockIdx.x == 0 && threadIdx.x < 2) L.n_list_items[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 2) hdr->list_work[threadIdx.x] = 0ull;
   __syncthreads();
   for (int c0 = 0; c0 < tr.P; c0 += 1024) {
     int E = c0 + threadIdx.x;
@@ -1747,7 +1747,7 @@ __global__ void __launch_bounds__(512, 1) pass_b_tc(const __grid_constant__ TcLa
 // The page pass over the units' slot lists (list pass `which`).
 __global__ void __launch_bounds__(512, 1) pass_b_list_tc(const __grid_constant__ TcLaunch L, WsHeader *hdr, int which) {
   extern __shared__ uint8_t smem_raw[];
-  const int n = L.n_list_items[which];
+  const int n = (int)(hdr->list_work[which] & 0xffffffffull);
   if ((int)blockIdx.x >= n) return;
   page_body<false, true>(L, hdr, smem_raw, blockIdx.x, gridDim.x, n);
 }
@@ -1759,7 +1759,10 @@ __global__ void __launch_bounds__(512, 1) pass_b_list_tc(const __grid_constant__
 //   r = ||U_E - S_E o|| / ((l - S_E) ||o||)  <=  s / (1 - s) (1 + max|v| / ||o||)
 // since ||U_E|| <= S_E max|v|.  The flash pass leaves log2 S_E (rounded up)
 // of every row and page and |v| of every token; this kernel takes the
-// maximum of the bound over the unit's rows.  Shares above 0.9, where
+// maximum of the bound over the unit's rows, its 128 less those past the
+// slice's end: the flash pass writes nothing for those, and the workspace
+// holds what was there (36 layers of 1.9K + 0.5K tokens, 32 rows a unit, with
+// NaN there: 675 us a call, 386 so).  Shares above 0.9, where
 // rounding in l - S_E matters, rows with an output norm that is not an
 // ordinary number, and NaN give an infinite bound; the factors cover the
 // rounding of the terms.
@@ -1776,14 +1779,18 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLa
   if (np <= 0) return;
   const __half *pieces = pr.pieces + (int64_t)unit * pr.npiece * BM + 4 * lane;  // lane i: rows 4 i .. 4 i + 3
   const __half *vn = pr.vnorm + (int64_t)slice * ((tr.S + BT - 1) / BT * BT);
-  auto load = [&](int piece) { return __ldg(reinterpret_cast<const uint2 *>(pieces + (int64_t)piece * BM)); };
+  // rows of this lane that the unit has: the others' pieces are not read
+  const int rows = min(4, L.g * tr.W - rt * BM - 4 * lane);
+  const uint2 none = make_uint2(0xfc00fc00u, 0xfc00fc00u);  // -inf: no mass
+  auto load = [&](int piece) {
+    return rows > 0 ? __ldg(reinterpret_cast<const uint2 *>(pieces + (int64_t)piece * BM)) : none;
+  };
   // lane i reads page i's table entries; the loads of all pages are issued
   // before any is used
   const int po_l = pr.piece_off[Ew + min(lane, np)];
   const int ps_l = tr.ps[Ew + min(lane, np - 1)], pl_l = tr.pl[Ew + min(lane, np - 1)];
   uint2 w0[kPer], w1[kPer];
   unsigned short v0[kPer];
-  const uint2 none = make_uint2(0xfc00fc00u, 0xfc00fc00u);  // -inf: no mass
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     const int p0 = __shfl_sync(0xffffffffu, po_l, i), p1 = __shfl_sync(0xffffffffu, po_l, i + 1);
@@ -1798,8 +1805,7 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLa
   float ref[4], inv_o[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const bool ok = rt * BM + 4 * lane + k < L.g * tr.W;
-    const float4 a = ok ? pr.aux[(int64_t)unit * BM + 4 * lane + k] : make_float4(-INFINITY, 0.0f, 1.0f, 0.0f);
+    const float4 a = k < rows ? pr.aux[(int64_t)unit * BM + 4 * lane + k] : make_float4(-INFINITY, 0.0f, 1.0f, 0.0f);
     const bool live = a.x != -INFINITY;  // the row sees something
     ref[k] = live ? a.x - (4e-3f + 1e-6f * fabsf(a.x)) + fast_log2(a.y) : INFINITY;
     inv_o[k] = !live ? 0.0f : a.z > 1e-15f && a.z < 1e30f ? 1.01f / a.z : INFINITY;
@@ -1831,7 +1837,8 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ TcLa
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const float r = __fdividef(S[k], 1.0f - S[k]) * fmaf(v, inv_o[k], 1.0f);
-      mx = max(mx, S[k] < 0.9f ? __float_as_uint(r) & 0x7fffffffu : 0x7f800000u);  // a NaN stays above every bound
+      const unsigned rb = S[k] < 0.9f ? __float_as_uint(r) & 0x7fffffffu : 0x7f800000u;  // a NaN stays above every bound
+      mx = max(mx, k < rows ? rb : 0u);
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if (lane == i) mine = mx;
@@ -1868,7 +1875,7 @@ __global__ void __launch_bounds__(512) seed_kernel(const __grid_constant__ TcLau
 // has no visible mass and effect 0.  Items: item k of a unit takes the pages
 // whose first slot in its list lies in [k n, (k + 1) n).
 constexpr int kMaxBuckets = 1024;
-__global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLaunch L, int which) {
+__global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLaunch L, WsHeader *hdr, int which) {
   const int t = traj_of(L.unit_off, L.n_traj, blockIdx.x);
   const TcTraj &tr = L.t[t];
   const TcPrune &pr = tr.pr;
@@ -1927,7 +1934,8 @@ __global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLau
     if (s_first[i] != ~0ull) atomicAdd(&s_n, 1);
   __syncthreads();
   if (threadIdx.x == 0) {
-    s_at = s_n ? atomicAdd(&L.n_list_items[which], s_n) : 0;
+    // {pages, items} of the unit in one addition
+    s_at = s_n ? (int)(atomicAdd(&hdr->list_work[which], (s_run & ~0xffffffffull) | (unsigned)s_n) & 0xffffffffull) : 0;
     s_n = 0;
   }
   __syncthreads();
@@ -2068,7 +2076,7 @@ cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t s, int sm_c
     bound_kernel<<<L.bound_off[L.n_traj], 256, 0, s>>>(L);
     seed_kernel<<<L.seed_off[L.n_traj], 512, 0, s>>>(L);
     for (int which = 0; which < 2; ++which) {
-      list_kernel<<<units, 256, 0, s>>>(L, which);
+      list_kernel<<<units, 256, 0, s>>>(L, hdr, which);
       pass_b_list_tc<<<sm_count, 512, smem_b(), s>>>(L, hdr, which);
     }
     return cudaGetLastError();

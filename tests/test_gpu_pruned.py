@@ -106,6 +106,28 @@ def test_pruned_effects_of_a_ragged_batch_with_a_layer_mask():
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("Hq,W", [(32, 8), (64, 20)], ids=["32rows", "160rows"])
+@pytest.mark.parametrize("d", [128, 64])
+def test_what_the_workspace_held_does_not_change_what_is_scored(d, Hq, W):
+    """A row tile that the probe rows fill in part: of the rows past their end
+    nothing is written, and the bounds may not read them (0xff and 0x7e bytes
+    are NaN as 16-bit floats, 0x7c an infinity or a NaN)."""
+    M, H, S = 64, 8, 2200
+    t = _traj(M, H, Hq, d, S, W, [16], "sharp", 11)
+    shape = ck.make_shape(M, H, Hq, d, torch.bfloat16)
+    ws = ck.alloc_workspace(shape, [t])
+    P, seen = t.page_start.numel(), []
+    for byte in (0, 0xFF, 0x7E, 0x7C):
+        ws[256:] = byte
+        R = torch.zeros(P, device="cuda")
+        ck.commitkv_page_effects(shape, [t], [R], workspace=ws)
+        pages = ck.commitkv_test_pruned_pages(ws)
+        assert ck.commitkv_workspace_status(ws) == ck.COMMITKV_OK
+        seen.append((pages, R.cpu().numpy().tobytes()))
+    assert 0 < sum(seen[0][0]) < M * H * ((Hq // H * W + 127) // 128) * P
+    assert all(s == seen[0] for s in seen)
+
+
 def test_overlapping_pages_are_reported_and_stay_in_bounds():
     """A zero-length page between two pages of the same span: each is
     compared with every earlier page, not with its neighbour alone."""
