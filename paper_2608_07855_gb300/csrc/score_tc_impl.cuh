@@ -1871,8 +1871,9 @@ __global__ void __launch_bounds__(512) seed_kernel(const __grid_constant__ TcLau
 
 // Writes the slot list of one unit per block and its work items.  Pass 0
 // takes the pages whose seed this unit is; pass 1, when R holds the seeds'
-// effects, the other pages whose bound is above R.  A page whose bound is 0
-// has no visible mass and effect 0.  Items: item k of a unit takes the pages
+// effects, the other pages whose bound is above R, or infinite: then the
+// effect may be a NaN, which the maximum ranks above an infinite R.  A page
+// whose bound is 0 has no visible mass and effect 0.  Items: item k of a unit takes the pages
 // whose first slot in its list lies in [k n, (k + 1) n).
 constexpr int kMaxBuckets = 1024;
 __global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLaunch L, WsHeader *hdr, int which) {
@@ -1901,7 +1902,7 @@ __global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLau
       if (which == 0) take = mine;
       else {
         const float b = pr.bound[(int64_t)unit * tr.P + E];
-        take = !mine && b != 0.0f && !(b <= tr.R[E]);
+        take = !mine && b != 0.0f && (!(b <= tr.R[E]) || b == INFINITY);
       }
       take = take && ns > 0;
     }

@@ -106,6 +106,20 @@ def test_pruned_effects_of_a_ragged_batch_with_a_layer_mask():
             assert np.array_equal(a, b)
 
 
+def test_a_nan_effect_ranks_above_an_infinite_one():
+    """The first page is all that the first window position sees (effect
+    infinite in every unit), and one head's values make its other rows'
+    effects NaN: a unit with an infinite bound is scored although R is
+    infinite already."""
+    t = _traj(128, 8, 16, 128, 1100, 64, [32], "normal", 5)
+    n = int(t.page_start[0] + t.page_len[0])
+    t.page_start[0], t.page_len[0] = 0, n
+    t.q_pos[0] = t.pos[n - 1]
+    t.v[0, 0, 3, 5] = float("inf")
+    pruned, full = _both([t], 128, 16)
+    assert np.isnan(full[0].view(np.float32)[0]) and np.array_equal(pruned[0], full[0])
+
+
 @pytest.mark.parametrize("Hq,W", [(32, 8), (64, 20)], ids=["32rows", "160rows"])
 @pytest.mark.parametrize("d", [128, 64])
 def test_what_the_workspace_held_does_not_change_what_is_scored(d, Hq, W):
