@@ -178,11 +178,15 @@ bool env_force_simt() {
   return e && (e[0] == 's' || e[0] == 'S');
 }
 
+// A cache that a scoring launch has work for: also one without pages, whose
+// row statistics the flash pass gives.
+bool active(const commitkv_traj &x) { return x.S > 0 && x.W > 0; }
+
 bool tc_eligible(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
   if (s->dtype != COMMITKV_BF16 || env_force_simt()) return false;
   for (int t = 0; t < n_traj; ++t) {
     const commitkv_traj &x = tr[t];
-    if (x.S == 0 || x.W == 0 || x.P == 0) continue;
+    if (!active(x)) continue;  // the others' tensor maps are encoded
     if (((uintptr_t)x.k | (uintptr_t)x.v | (uintptr_t)x.q) % 16) return false;
     if ((x.stride_tok * 2) % 16 || (x.stride_head * 2) % 16 || (x.stride_layer * 2) % 16) return false;
     if (x.stride_head == 0 || x.stride_layer == 0) return false;
@@ -564,15 +568,15 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       tt.nchunk = c.nchunk;
       tt.nrt = c.nrt;
       tt.nbitem = c.nbitem;
-      bool active = x.S > 0 && x.W > 0;
-      int ia = active ? nl * shape->kv_heads * c.nchunk * c.nrt : 0;
-      int ib = active && x.P > 0 ? nl * shape->kv_heads * c.nbitem * c.nrt : 0;
+      const bool act = active(x);
+      int ia = act ? nl * shape->kv_heads * c.nchunk * c.nrt : 0;
+      int ib = act && x.P > 0 ? nl * shape->kv_heads * c.nbitem * c.nrt : 0;
       T.item_off_a[i + 1] = T.item_off_a[i] + ia;
       T.item_off_b[i + 1] = T.item_off_b[i] + ib;
-      T.row_off[i + 1] = T.row_off[i] + (active ? nl * shape->kv_heads * L.batch.g * x.W : 0);
-      T.slice_off[i + 1] = T.slice_off[i] + (active ? nl * shape->kv_heads : 0);
-      T.unit_off[i + 1] = T.unit_off[i] + (active && x.P > 0 ? nl * shape->kv_heads * c.nrt : 0);
-      if (active && !tc::build_maps(d, T.maps[i], L.batch.t[t], shape->layers, shape->kv_heads, shape->q_heads))
+      T.row_off[i + 1] = T.row_off[i] + (act ? nl * shape->kv_heads * L.batch.g * x.W : 0);
+      T.slice_off[i + 1] = T.slice_off[i] + (act ? nl * shape->kv_heads : 0);
+      T.unit_off[i + 1] = T.unit_off[i] + (act && x.P > 0 ? nl * shape->kv_heads * c.nrt : 0);
+      if (act && !tc::build_maps(d, T.maps[i], L.batch.t[t], shape->layers, shape->kv_heads, shape->q_heads))
         return COMMITKV_ERR_CUDA;
     }
     // one array of work items for the launch, after its trajectories' regions

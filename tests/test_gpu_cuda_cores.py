@@ -68,3 +68,40 @@ def test_infinite_value_row_stays_in_its_head():
     g = cfg.Hq // cfg.H
     assert np.array_equal(out[0][:, g:], out[1][:, g:])
     assert np.isfinite(out[0]).any()
+
+
+@pytest.mark.parametrize("off", ["pointer", "head stride"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_pageless_cache_that_the_tensor_cores_cannot_read(d, off, monkeypatch):
+    """The flash pass reads a cache without pages too (its row statistics): one
+    element off a 16-byte boundary, or one head for all KV heads, sends its
+    batch to the CUDA cores, as a cache with pages does."""
+    M, H, S, W = 2, 2, 300, 8
+    gen = torch.Generator("cuda").manual_seed(d)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    pos = torch.arange(S, **i32)
+
+    def cache(odd, pages):
+        def values():
+            flat = torch.randn(M * H * S * d + 1, generator=gen, device="cuda").bfloat16()
+            if odd and off == "head stride":
+                return flat[:M * S * d].view(M, 1, S, d).expand(M, H, S, d)
+            return flat[int(odd):][:M * H * S * d].view(M, H, S, d)
+        Q = torch.randn(M, 4, W, d, generator=gen, device="cuda").bfloat16()
+        ps = torch.arange(0, 280 if pages else 0, 20, **i32)
+        return ck.TrajTensors(values(), values(), pos, Q, pos[-W:].contiguous(), ps, torch.full_like(ps, 16))
+
+    trajs = [cache(False, True), cache(True, False)]
+    shape = ck.make_shape(M, H, 4, d, torch.bfloat16)
+    ws = ck.alloc_workspace(shape, trajs)
+    out = []
+    for path in ("tc", "simt"):
+        monkeypatch.setenv("COMMITKV_SCORING", path)
+        R = [torch.zeros(t.page_start.numel(), device="cuda") for t in trajs]
+        stats = torch.zeros(M, 4, W, d + 4, device="cuda")
+        ck.commitkv_page_effects(shape, trajs, R, workspace=ws)
+        ck.commitkv_page_effects(shape, trajs[1:], R[1:], stats_out=[stats], workspace=ws)
+        assert ck.commitkv_workspace_status(ws) == ck.COMMITKV_OK
+        out.append((R[0], stats))
+    assert out[0][0].max() > 0 and torch.equal(out[0][0], out[1][0])
+    assert out[0][1][..., 2].min() > 0 and torch.equal(out[0][1], out[1][1])
