@@ -967,8 +967,10 @@ __device__ __forceinline__ void merge_row(const TcLaunch &L, int t, int li, int 
   }
 }
 
-// One warp per probe row of the selected layers (the two-launch path).
-__global__ void __launch_bounds__(256) combine_tc(const __grid_constant__ TcLaunch L) {
+// One warp per probe row of the selected layers (the two-launch path).  Four
+// blocks a SM: two registers above 64 a thread leave three (36,864 rows of
+// 16 chunks: 35 us, 30 so).
+__global__ void __launch_bounds__(256, 4) combine_tc(const __grid_constant__ TcLaunch L) {
   const int gw = (blockIdx.x * 256 + threadIdx.x) / 32, lane = threadIdx.x % 32;
   if (gw >= L.row_off[L.n_traj]) return;
   const int t = traj_of(L.row_off, L.n_traj, gw);
