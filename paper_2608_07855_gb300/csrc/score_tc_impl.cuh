@@ -1884,9 +1884,17 @@ __global__ void __launch_bounds__(512) seed_kernel(const __grid_constant__ TcLau
 // effects, the other pages whose bound is above R, or infinite: then the
 // effect may be a NaN, which the maximum ranks above an infinite R.  A page
 // whose bound is 0 has no visible mass and effect 0.  Items: item k of a unit takes the pages
-// whose first slot in its list lies in [k n, (k + 1) n).
+// whose first slot in its list lies in [k n, (k + 1) n).  A unit that keeps half
+// of the slots or more takes twice as many an item, as the full page pass does,
+// where that leaves kPairedPerSm items a SM: every item costs its start.
+// Nothing dropped, 36 layers of 18K tokens (2,592 such items) in pages of 100
+// and 250: page pass 833 us, 784 so, and in pages of 16 1,495 and 1,443;
+// with 576 items a call takes longer (2.4K tokens, 32 rows: 431 us, 469 to 585
+// paired; 16 layers of 64 channels, 9.2K: 613 and 660), and so does one whose
+// units keep little (all paired, 16K + 2K with a sixth kept: page pass 248 us, 298).
+constexpr int kPairedPerSm = 8;
 constexpr int kMaxBuckets = 1024;
-__global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLaunch L, WsHeader *hdr, int which) {
+__global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLaunch L, WsHeader *hdr, int which, int sm_count) {
   const int t = traj_of(L.unit_off, L.n_traj, blockIdx.x);
   const TcTraj &tr = L.t[t];
   const TcPrune &pr = tr.pr;
@@ -1941,6 +1949,15 @@ __global__ void __launch_bounds__(256) list_kernel(const __grid_constant__ TcLau
     __syncthreads();
   }
   const unsigned long long all = ((s_run & 0xffffffffull) << 32) | (s_run >> 32);  // {slots, pages}
+  const int64_t slots = tr.slot_off[tr.P];
+  if (2 * (int64_t)(s_run & 0xffffffffull) >= slots &&
+      gridDim.x * slots >= (int64_t)kPairedPerSm * sm_count * 2 * kListSlotsPerItem) {
+    for (int i = 2 * threadIdx.x; i + 1 < nbuckets; i += 512) {  // the smaller entry: the earlier pages
+      s_first[i] = min(s_first[i], s_first[i + 1]);
+      s_first[i + 1] = ~0ull;
+    }
+    __syncthreads();
+  }
   for (int i = threadIdx.x; i < nbuckets; i += 256)
     if (s_first[i] != ~0ull) atomicAdd(&s_n, 1);
   __syncthreads();
@@ -2087,7 +2104,7 @@ cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t s, int sm_c
     bound_kernel<<<L.bound_off[L.n_traj], 256, 0, s>>>(L);
     seed_kernel<<<L.seed_off[L.n_traj], 512, 0, s>>>(L);
     for (int which = 0; which < 2; ++which) {
-      list_kernel<<<units, 256, 0, s>>>(L, hdr, which);
+      list_kernel<<<units, 256, 0, s>>>(L, hdr, which, sm_count);
       pass_b_list_tc<<<sm_count, 512, smem_b(), s>>>(L, hdr, which);
     }
     return cudaGetLastError();
