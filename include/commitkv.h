@@ -122,10 +122,17 @@ typedef struct {
   float tau_use, tau_dead, rho_use, rho_dead;
 } commitkv_thresholds;
 
-/* Size in bytes of the workspace every entry point below needs for these
- * trajectories (the maximum over the calls).  Pass the largest caches the
- * workspace will serve (normally the post-commit ones).  Returns 0 for
- * invalid arguments. */
+/* Size in bytes of the workspace with which every entry point below runs at
+ * its best for these trajectories (the maximum over the calls).  Pass the
+ * largest caches the workspace will serve (normally the post-commit ones).
+ * Returns 0 for invalid arguments.
+ * The scoring calls also take a smaller workspace, down to their row
+ * statistics and per-chunk partial results, and run slower in it: large bf16
+ * calls then score every page (the same effects; the tables for skipping
+ * pages take up to 256 bytes per page and 128-token piece of it in every row
+ * tile of 128 probe rows), 64-channel bf16 calls and small fp32 calls use
+ * fewer or other blocks (effects within a few 1e-6).  Below that they return
+ * COMMITKV_ERR_WORKSPACE. */
 size_t commitkv_workspace_size(const commitkv_shape *shape, int32_t n_traj,
                                const commitkv_traj *trajs);
 

@@ -5,6 +5,9 @@
 
 #include <stdlib.h>
 
+#include <algorithm>
+#include <functional>
+
 #include "ckv_internal.cuh"
 #include "score_tc.cuh"
 
@@ -136,14 +139,21 @@ int64_t simt_units(const commitkv_shape *s, int n_layers, int n_traj, const comm
 
 // A call that gives few blocks takes shorter chunks, down to 128 tokens, as
 // long as they stay below this number (the fp32 Tiny workload, 18 blocks of
-// 512 tokens: pass A 161 us; 72 blocks of 128: 18 us with the merge of eight rows); larger calls at most 16
+// 512 tokens: pass A 161 us; 72 blocks of 128: 18 us with the merge of eight rows) and
+// their partials fit the scratch; other calls at most 16
 // chunks per (layer, KV head), at least 512 tokens each.
 constexpr int64_t kSimtMaxSmallUnits = 1024;
 constexpr int kSimtMinChunk = 128;
 
-int chunk_len_for(const commitkv_shape *s, int n_layers, int n_traj, const commitkv_traj *tr) {
-  for (int c = kSimtMinChunk; c < 512; c *= 2)
-    if (simt_units(s, n_layers, n_traj, tr, c) <= kSimtMaxSmallUnits) return c;
+size_t simt_bytes(const commitkv_shape *s, size_t units) {
+  return align_up(units * simt_rows_per_block() * (s->head_dim + 4) * 4);
+}
+
+int chunk_len_for(const commitkv_shape *s, int n_layers, int n_traj, const commitkv_traj *tr, size_t scratch) {
+  for (int c = kSimtMinChunk; c < 512; c *= 2) {
+    const int64_t units = simt_units(s, n_layers, n_traj, tr, c);
+    if (units <= kSimtMaxSmallUnits && simt_bytes(s, (size_t)units) <= scratch) return c;
+  }
   int smax = 0;
   for (int t = 0; t < n_traj; ++t) smax = tr[t].S > smax ? tr[t].S : smax;
   int c = (smax + 15) / 16;
@@ -207,12 +217,17 @@ int simt_chunk_bound(int S) {
 }
 
 // Partials of the CUDA-core path for these caches or smaller ones, in units of
-// a block's rows.
-size_t simt_unit_bound(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+// a block's rows: with the long chunks, which it can always take, and with
+// those of small calls as well.
+size_t simt_unit_floor(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
   const int g = s->q_heads / s->kv_heads;
   size_t units = 0;
   for (int t = 0; t < n_traj; ++t)
     units += (size_t)s->layers * s->kv_heads * simt_chunk_bound(tr[t].S) * cdiv(g * tr[t].W, simt_rows_per_block());
+  return units;
+}
+size_t simt_unit_bound(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  const size_t units = simt_unit_floor(s, n_traj, tr);
   const int64_t small = simt_units(s, s->layers, n_traj, tr, kSimtMinChunk);
   const size_t few = (size_t)(small < kSimtMaxSmallUnits ? small : kSimtMaxSmallUnits);
   return units > few ? units : few;
@@ -227,23 +242,28 @@ bool env_fused() {
   return e && e[0] == '1';
 }
 
+// (unit, token) pairs of a cache.
+int64_t prune_work(const commitkv_shape *s, int n_layers, const commitkv_traj &x) {
+  return (int64_t)n_layers * s->kv_heads * cdiv(s->q_heads / s->kv_heads * x.W, tc::kRowsPerTile) * x.S;
+}
+
 // Whether the page pass of a launch scores only the pages whose bound can
 // raise R (exact; see bound_kernel).  It needs
 // R alone as output: the maxima per head take every page of every head.
-bool prune_pages(int n, const commitkv_traj *tr, int slices, int g, float *const *headR) {
+bool prune_pages(const commitkv_shape *s, int n_layers, int n, const commitkv_traj *tr, float *const *headR) {
   int64_t work = 0;
   for (int t = 0; t < n; ++t) {
     if (headR[t]) return false;
-    if (tr[t].S == 0 || tr[t].W == 0 || tr[t].P == 0) continue;
+    if (!active(tr[t]) || tr[t].P == 0) continue;
     if ((int64_t)tr[t].P * tc::kMinPageTokens > tr[t].S) return false;
-    work += (int64_t)slices * cdiv(g * tr[t].W, tc::kRowsPerTile) * tr[t].S;
+    work += prune_work(s, n_layers, tr[t]);
   }
   return work >= tc::kMinPruneWork;
 }
 
 // Flash-pass partial slots the tensor-core path may need for these caches or
 // smaller ones: one per item of the two-launch chunking, or the fused
-// launch's ring (at most kMaxFusedCtas x kPartialRing slots, and at most one
+// launch's ring (128 channels; at most kMaxFusedCtas x kPartialRing slots, and at most one
 // per item of its chunking: about kFusedItemsPerSlice items per slice).
 size_t tc_partial_slots(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
   size_t items = 0, fused = 0;
@@ -254,34 +274,67 @@ size_t tc_partial_slots(const commitkv_shape *s, int n_traj, const commitkv_traj
   }
   const size_t ring = (size_t)tc::kMaxFusedCtas * tc::kPartialRing;
   if (fused > ring) fused = ring;
+  if (s->head_dim != 128) fused = 0;
   return items > fused ? items : fused;
 }
 
+// The tensor-core path without the pruned page pass.
 size_t tc_score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
   size_t slots = 0, slices = 0;
   for (int t = 0; t < n_traj; ++t) {
     TcCounts c = tc_counts(s, tr[t], tc_chunk_len(1, &tr[t]));
     slots += align_up((size_t)(tr[t].P + 1) * 4) + align_up((size_t)c.nbitem * 32) + kAlign +
              align_up(((size_t)cdiv(tr[t].S, 16) + tr[t].P) * 16);
-    slots += tc::prune_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt) +
-             align_up(tc::prune_item_bytes(tr[t].S, tr[t].P, s->layers * s->kv_heads, c.nrt));
     slices += (size_t)s->layers * s->kv_heads;
   }
   return align_up(tc_partial_slots(s, n_traj, tr) * tc::kPartsPerItem * tc::kRowsPerTile * (s->head_dim + 4) * 4) +
          align_up(slices * 2 * tc::kCounterStride * 4) + slots;
 }
 
-// Region sizes of each call (bytes after the 256-byte header).
-size_t score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
-  int RB = simt_rows_per_block(), d = s->head_dim;
-  size_t stats = 0;
+// What the pruned page pass adds for one trajectory; the launches of a call
+// use one region after another.
+size_t prune_traj_bytes(const commitkv_shape *s, const commitkv_traj &x) {
+  const int slices = s->layers * s->kv_heads, nrt = tc_counts(s, x, tc_chunk_len(1, &x)).nrt;
+  return tc::prune_bytes(x.S, x.P, slices, nrt) + align_up(tc::prune_item_bytes(x.S, x.P, slices, nrt));
+}
+
+// The region for any launch of up to kMaxTc of these trajectories, none where
+// no such launch has the work for pruning.
+size_t prune_region_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  size_t bytes[kMaxTraj];
+  int64_t work = 0;
   for (int t = 0; t < n_traj; ++t) {
-    stats += align_up((size_t)s->layers * s->q_heads * tr[t].W * (d + 4) * 4) + align_up((size_t)tr[t].W * 4);
+    bytes[t] = prune_traj_bytes(s, tr[t]);
+    work += prune_work(s, s->layers, tr[t]);
   }
-  size_t scratch = align_up(simt_unit_bound(s, n_traj, tr) * RB * (d + 4) * 4);
-  const size_t tcb = tc_score_bytes(s, n_traj, tr);
-  if (tcb > scratch) scratch = tcb;
-  return scratch + stats;
+  if (work < tc::kMinPruneWork) return 0;
+  std::sort(bytes, bytes + n_traj, std::greater<size_t>());
+  size_t sum = 0;
+  for (int t = 0; t < n_traj && t < tc::kMaxTc; ++t) sum += bytes[t];
+  return sum;
+}
+
+// Scoring calls, bytes after the 256-byte header: first the row statistics
+// and visible counts, then the scratch of the path taken.  With the larger
+// size a call takes its fastest path; from the smaller one on it runs, on the
+// path that the scratch has room for: the full page pass (the same effects),
+// the CUDA cores (64 channels), longer chunks there.
+size_t stats_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  size_t b = 0;
+  for (int t = 0; t < n_traj; ++t)
+    b += align_up((size_t)s->layers * s->q_heads * tr[t].W * (s->head_dim + 4) * 4) + align_up((size_t)tr[t].W * 4);
+  return b;
+}
+size_t score_bytes_min(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  size_t scratch = simt_bytes(s, simt_unit_floor(s, n_traj, tr));
+  if (s->dtype == COMMITKV_BF16 && s->head_dim == 128) scratch = std::max(scratch, tc_score_bytes(s, n_traj, tr));
+  return stats_bytes(s, n_traj, tr) + scratch;
+}
+size_t score_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr) {
+  size_t scratch = simt_bytes(s, simt_unit_bound(s, n_traj, tr));
+  if (s->dtype == COMMITKV_BF16)
+    scratch = std::max(scratch, tc_score_bytes(s, n_traj, tr) + prune_region_bytes(s, n_traj, tr));
+  return stats_bytes(s, n_traj, tr) + scratch;
 }
 
 size_t joint_bytes(const commitkv_shape *s, int n_traj, const commitkv_traj *tr, int n_layers) {
@@ -413,8 +466,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   // with both kinds of trajectories is split.
   const bool simt64 = shape->head_dim == 64 && shape->dtype == COMMITKV_BF16 && (from_stats || n_stats > 0);
   if (simt64 && !from_stats && n_stats < n_traj) {
-    const size_t all = kAlign + score_bytes(shape, n_traj, trajs);
-    if ((st = check_ws(workspace, workspace_bytes, all))) return st;
+    if ((st = check_ws(workspace, workspace_bytes, kAlign + score_bytes_min(shape, n_traj, trajs)))) return st;
     for (int with = 0; with < 2; ++with) {
       commitkv_traj tr[COMMITKV_MAX_TRAJ];
       float *R[COMMITKV_MAX_TRAJ], *hR[COMMITKV_MAX_TRAJ], *so[COMMITKV_MAX_TRAJ];
@@ -438,10 +490,10 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   memset(&L, 0, sizeof L);
   fill_batch(L.batch, shape, n_traj, trajs, layer_mask);
   int nl = L.batch.n_layers;
-  size_t need = kAlign + score_bytes(shape, n_traj, trajs);
-  if ((st = check_ws(workspace, workspace_bytes, need))) return st;
+  if ((st = check_ws(workspace, workspace_bytes, kAlign + score_bytes_min(shape, n_traj, trajs)))) return st;
+  const size_t stats_size = stats_bytes(shape, n_traj, trajs), scratch = workspace_bytes - kAlign - stats_size;
 
-  int CL = chunk_len_for(shape, nl, n_traj, trajs), RB = simt_rows_per_block(), PG = simt_pages_per_block();
+  int CL = chunk_len_for(shape, nl, n_traj, trajs, scratch), RB = simt_rows_per_block(), PG = simt_pages_per_block();
   // small calls: fewer pages per block, down to one, until there is a block
   // per SM (half as many blocks, this line, twice as many: 2K tokens of one
   // layer and two heads 24, 24 and 30 us; two layers of four heads, 1.5K
@@ -455,7 +507,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   L.pages_per_block = PG;
   int g = L.batch.g, d = shape->head_dim;
   L.chunk_len = CL;
-  char *base = static_cast<char *>(workspace) + kAlign;
+  char *sbase = static_cast<char *>(workspace) + kAlign, *base = sbase + stats_size;
   for (int t = 0; t < n_traj; ++t) {
     int rows = g * trajs[t].W;
     L.nrb[t] = cdiv(rows, RB);
@@ -466,12 +518,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     L.row_off[t + 1] = L.row_off[t] + nl * shape->kv_heads * rows;
   }
   float *partials = reinterpret_cast<float *>(base);
-  // scratch (either path's partials) first, then the stats of trajectories
-  // without stats_out; the layout is computed for every layer
-  size_t scratch = align_up(simt_unit_bound(shape, n_traj, trajs) * RB * (d + 4) * 4);
-  const size_t tcb = tc_score_bytes(shape, n_traj, trajs);
-  if (tcb > scratch) scratch = tcb;
-  char *sbase = base + scratch;
+  // the statistics' layout is computed for every layer
   for (int t = 0; t < n_traj; ++t) {
     size_t sb = align_up((size_t)shape->layers * shape->q_heads * trajs[t].W * (d + 4) * 4);
     if (from_stats) L.stats[t] = const_cast<float *>(stats_in[t]);  // read only
@@ -492,7 +539,8 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     if (e != cudaSuccess) return cuda_status(e);
   }
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
-  if (!tc_eligible(shape, n_traj, trajs) || simt64)
+  const size_t tcb = tc_score_bytes(shape, n_traj, trajs);
+  if (!tc_eligible(shape, n_traj, trajs) || simt64 || tcb > scratch)
     return cuda_status(launch_score_simt(L, partials, hdr, stream));
   // tensor-core path: trajectories in launches of up to tc::kMaxTc
   static thread_local tc::TcLaunch T;
@@ -520,7 +568,12 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   for (int b0 = 0; b0 < n_traj; b0 += tc::kMaxTc) {
     int nb = n_traj - b0 < tc::kMaxTc ? n_traj - b0 : tc::kMaxTc;
     memset(&T, 0, sizeof T);
-    T.prune = !fused && !from_stats && prune_pages(nb, trajs + b0, nl * shape->kv_heads, L.batch.g, L.headR + b0);
+    // after the launches' own regions, one for all of them
+    char *prune_base = base + tcb;
+    size_t prune_size = 0;
+    for (int i = 0; i < nb; ++i) prune_size += prune_traj_bytes(shape, trajs[b0 + i]);
+    T.prune = !fused && !from_stats && prune_size <= scratch - tcb &&
+              prune_pages(shape, nl, nb, trajs + b0, L.headR + b0);
     T.n_traj = nb;
     T.M = shape->layers;
     T.H = shape->kv_heads;
@@ -553,10 +606,10 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       slot_base += kAlign;
       tt.slot_tab = reinterpret_cast<int4 *>(slot_base);
       slot_base += align_up(((size_t)cdiv(x.S, 16) + x.P) * 16);
-      {
+      if (T.prune) {
         const int slices = shape->layers * shape->kv_heads;
-        if (T.prune) tc::prune_layout(tt.pr, slot_base, x.S, x.P, slices, c.nrt);
-        slot_base += tc::prune_bytes(x.S, x.P, slices, c.nrt);
+        tc::prune_layout(tt.pr, prune_base, x.S, x.P, slices, c.nrt);
+        prune_base += tc::prune_bytes(x.S, x.P, slices, c.nrt);
       }
       tt.stats = L.stats[t];
       tt.nvis_w = L.nvis_w[t];
@@ -579,11 +632,8 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
       if (act && !tc::build_maps(d, T.maps[i], L.batch.t[t], shape->layers, shape->kv_heads, shape->q_heads))
         return COMMITKV_ERR_CUDA;
     }
-    // one array of work items for the launch, after its trajectories' regions
-    T.list_items = reinterpret_cast<int4 *>(slot_base);
-    for (int i = 0; i < nb; ++i)
-      slot_base += align_up(tc::prune_item_bytes(trajs[b0 + i].S, trajs[b0 + i].P, shape->layers * shape->kv_heads,
-                                                 T.t[i].nrt));
+    // one array of work items for the launch, after its trajectories' parts
+    if (T.prune) T.list_items = reinterpret_cast<int4 *>(prune_base);
     e = tc::launch_score_tc(d, T, hdr, stream, sms);
     if (e != cudaSuccess) return cuda_status(e);
   }

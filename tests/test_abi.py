@@ -147,6 +147,19 @@ def test_joint_and_variant_validation(lib):
               None) == ck.COMMITKV_ERR_INVALID_ARG
 
 
+def test_workspace_holds_what_a_call_can_use(lib):
+    """The tables for skipping pages are sized for bf16 caches with the work
+    for it: not for fp32 ones, whose path keeps nothing per page, nor for
+    small calls."""
+    def size(dtype, M, S, P):
+        shape = ck.Shape(M, 8, 32, 128, dtype, 0.0)
+        return lib.commitkv_workspace_size(ctypes.byref(shape), 1, (ck.Traj * 1)(_good_traj(S=S, W=32, P=P, H=8)))
+
+    assert size(ck.COMMITKV_F32, 32, 16384, 8192) == size(ck.COMMITKV_F32, 32, 16384, 16)
+    assert size(ck.COMMITKV_BF16, 2, 2000, 1000) - size(ck.COMMITKV_BF16, 2, 2000, 10) < 1000 * 64
+    assert size(ck.COMMITKV_BF16, 32, 16384, 8192) - size(ck.COMMITKV_BF16, 32, 16384, 16) > 8000 * 32 * 8 * 256
+
+
 def test_workspace_covers_smaller_caches(lib):
     """A workspace sized for the post-commit caches serves the pre-commit
     call too (its S and P are smaller), for every chunking regime."""

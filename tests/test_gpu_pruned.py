@@ -106,6 +106,41 @@ def test_pruned_effects_of_a_ragged_batch_with_a_layer_mask():
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("M,H,Hq,d,dtype,S,W,P,size", [(64, 8, 32, 128, "bfloat16", 2200, 8, 130, 112596992),
+                                                       (16, 2, 8, 64, "bfloat16", 2200, 8, 130, 3064320),
+                                                       (1, 2, 4, 64, "float32", 2300, 16, 140, 192000)],
+                         ids=["pruned", "64channels", "small-f32"])
+def test_a_workspace_without_room_for_the_faster_path(M, H, Hq, d, dtype, S, W, P, size):
+    """`size` is what commitkv_workspace_size gave before there were bounds,
+    64-channel tensor-core kernels and short chunks of small calls: such a
+    buffer still serves, and a quarter of it is refused as before."""
+    t = _traj(M, H, Hq, d, S, W, [16], "normal", 7)
+    dt = getattr(torch, dtype)
+    t = ck.TrajTensors(t.k.to(dt), t.v.to(dt), t.pos, t.q.to(dt), t.q_pos, t.pos[:0].new_tensor(range(0, 16 * P, 16)),
+                       t.pos.new_full((P,), 16))
+    shape = ck.make_shape(M, H, Hq, d, dt)
+    out = []
+    for n in (ck.commitkv_workspace_size(shape, [t]), size):
+        ws = torch.empty(n + 512, dtype=torch.uint8, device="cuda")
+        ws[n:] = 0x5A  # past the end
+        ck.commitkv_workspace_init(ws[:n])
+        R = torch.zeros(P, device="cuda")
+        ck.commitkv_page_effects(shape, [t], [R], workspace=ws[:n])
+        pages = ck.commitkv_test_pruned_pages(ws[:n])
+        assert ck.commitkv_workspace_status(ws[:n]) == ck.COMMITKV_OK
+        assert bool((ws[n:] == 0x5A).all())
+        out.append((n, pages, R))
+    assert out[0][0] > size
+    assert (sum(out[0][1]) > 0) == (d == 128) and sum(out[1][1]) == 0
+    a, b = out[0][2], out[1][2]
+    if d == 128:  # the same values
+        assert torch.equal(a, b)
+    else:  # each within 1e-4 of the exact effects (the bound of both paths' tests)
+        assert torch.isfinite(a).all() and ((a - b).abs() <= 2e-4 * a).all()
+    with pytest.raises(RuntimeError):
+        ck.commitkv_page_effects(shape, [t], [R], workspace=torch.empty(size // 4 // 256 * 256, dtype=torch.uint8, device="cuda"))
+
+
 def test_a_nan_effect_ranks_above_an_infinite_one():
     """The first page is all that the first window position sees (effect
     infinite in every unit), and one head's values make its other rows'
