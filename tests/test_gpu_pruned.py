@@ -71,10 +71,15 @@ CASES = [
     (64, 8, 16, 4, 3000, [2800], "sharp"),  # one page of many tiles holding almost everything
     (64, 8, 16, 8, 2100, [2, 3], "normal"),
     (64, 8, 16, 8, 2100, [1, 2], "normal"),  # pages too short to prune: the full pass both times
+    (256, 16, 32, 32, 700, [16], "uniform"),  # units that keep everything, enough of them for items of two buckets
+    (128, 16, 32, 32, 1500, [16], "uniform"),  # the same with a third bucket alone
 ]
 
 
-def _both(trajs, M, Hq, mask=None):
+def _both(trajs, M, Hq, mask=None, prunes=True, most=1.0):
+    """R with the pruned page pass and with the full one, as bits.  `prunes`:
+    whether the first call prunes; then at most the share `most` of the (row
+    tile, page) pairs is scored."""
     shape = ck.make_shape(M, trajs[0].k.shape[1], Hq, trajs[0].k.shape[3], torch.bfloat16)
     ws = ck.alloc_workspace(shape, trajs)
     out = []
@@ -82,6 +87,10 @@ def _both(trajs, M, Hq, mask=None):
         R = [torch.full((t.page_start.numel(),), -1.0, device="cuda") for t in trajs]
         hR = [torch.zeros(M, Hq, t.page_start.numel(), device="cuda") for t in trajs] if head else None
         ck.commitkv_page_effects(shape, trajs, R, head_R_out=hR, layer_mask=mask, workspace=ws)
+        scored = sum(ck.commitkv_test_pruned_pages(ws))
+        tiles = [-(-Hq // shape.kv_heads * t.q.shape[2] // 128) * t.page_start.numel() for t in trajs]
+        assert (scored > 0) == (prunes and not head)
+        assert scored <= most * M * shape.kv_heads * sum(tiles)
         assert ck.commitkv_workspace_status(ws) == ck.COMMITKV_OK
         out.append([r.cpu().numpy().view(np.uint32) for r in R])
     return out
@@ -91,7 +100,12 @@ def _both(trajs, M, Hq, mask=None):
 @pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[6]}-{c[4]}-{c[5][0]}")
 def test_pruned_effects_equal_the_full_pass(case, d):
     M, H, Hq, W, S, sizes, kind = case
-    pruned, full = _both([_traj(M, H, Hq, d, S, W, sizes, kind, d + 1)], M, Hq)
+    short = sizes == [1, 2]
+    t = _traj(M, H, Hq, d, S, W, sizes, kind, d + 1, 0 if short else 60)
+    assert (2 * t.page_start.numel() > S) == short
+    # a fifth to three fifths is scored of the sharp caches with many pages, a hundredth of short pages
+    most = 0.75 if kind == "sharp" and len(t.page_start) > 1 else 0.05 if sizes == [2, 3] else 1.0
+    pruned, full = _both([t], M, Hq, prunes=not short, most=most)
     assert np.array_equal(pruned[0], full[0])
 
 
