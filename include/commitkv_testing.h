@@ -36,6 +36,10 @@ commitkv_status commitkv_test_barrier_timeout(void *workspace, size_t workspace_
 commitkv_status commitkv_test_pruned_pages(const void *workspace, size_t workspace_bytes, uint64_t *pages_out,
                                            cudaStream_t stream);
 
+/* Kernels that the calling thread's calls have launched so far (a counter per
+ * thread, which nothing else reads). */
+uint64_t commitkv_test_launches(void);
+
 #ifdef __cplusplus
 }
 #endif

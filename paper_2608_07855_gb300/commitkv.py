@@ -99,6 +99,8 @@ def load_library(build_if_missing: bool = True) -> ctypes.CDLL:
                                              i32, vp, vp, vp, vp, vp, vp, vp]
     lib.commitkv_test_barrier_timeout.argtypes = [vp, sz, i32, vp]
     lib.commitkv_test_pruned_pages.argtypes = [vp, sz, vp, vp]
+    lib.commitkv_test_launches.argtypes = []
+    lib.commitkv_test_launches.restype = ctypes.c_uint64
     lib.commitkv_token_scores.argtypes = [P(Shape), i32, P(Traj), vp, vp, vp, vp, sz, vp]
     for f in ("commitkv_workspace_init", "commitkv_workspace_status", "commitkv_page_effects",
               "commitkv_page_effects_from_stats", "commitkv_classify", "commitkv_classify_variant",
@@ -268,6 +270,11 @@ def commitkv_test_pruned_pages(ws, stream=None):
     _check(load_library().commitkv_test_pruned_pages(_ptr(ws), ws.numel(), out, _stream(stream)),
            "commitkv_test_pruned_pages")
     return out[0], out[1]
+
+
+def commitkv_test_launches() -> int:
+    """Kernels that this thread's calls have launched so far."""
+    return load_library().commitkv_test_launches()
 
 
 def commitkv_page_effects(shape: Shape, trajs, R_out, head_R_out=None, stats_out=None,

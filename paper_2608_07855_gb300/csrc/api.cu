@@ -21,6 +21,11 @@ int simt_rows_per_block();
 int simt_pages_per_block();
 int compact_max_pending();
 
+uint64_t &launch_count() {
+  static thread_local uint64_t n = 0;
+  return n;
+}
+
 commitkv_status check_shape(const commitkv_shape *s) {
   if (!s) return COMMITKV_ERR_INVALID_ARG;
   if (s->layers < 1 || s->layers > kMaxLayers || s->kv_heads < 1 || s->q_heads < s->kv_heads ||
@@ -409,6 +414,8 @@ commitkv_status commitkv_workspace_status(const void *workspace, size_t workspac
   }
   return (commitkv_status)h.status;
 }
+
+uint64_t commitkv_test_launches(void) { return launch_count(); }
 
 commitkv_status commitkv_test_pruned_pages(const void *workspace, size_t workspace_bytes, uint64_t *pages_out,
                                            cudaStream_t stream) {

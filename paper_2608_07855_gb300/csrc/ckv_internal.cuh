@@ -110,6 +110,10 @@ commitkv_status check_compact_args(const commitkv_shape *s, int32_t n_traj, cons
                                    int32_t pending_tokens_BN, int32_t pending_cap_pages,
                                    int32_t *const *idx_out, const int32_t *n_idx_out);
 
+// Kernels launched by the calling thread so far (commitkv_test_launches): every
+// launch adds to it.
+uint64_t &launch_count();
+
 // Launch helpers implemented in the .cu files ------------------------------
 
 struct ScoreLaunch {

@@ -147,10 +147,12 @@ cudaError_t launch_classify(const ClassifyLaunch &L, WsHeader *hdr, cudaStream_t
   if (pmax > 0) {
     dim3 grid((pmax + kPagesPerBlock - 1) / kPagesPerBlock, L.n_traj);
     classify_state_kernel<<<grid, kThreads, 0, stream>>>(L, hdr);
+    ++launch_count();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   classify_order_kernel<<<L.n_traj, kThreads, 0, stream>>>(L);
+  ++launch_count();
   return cudaGetLastError();
 }
 

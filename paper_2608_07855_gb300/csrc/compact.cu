@@ -442,6 +442,7 @@ cudaError_t launch_compact(const CompactLaunch &L, WsHeader *hdr, cudaStream_t s
   cfg.stream = stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
+  ++launch_count();
   cudaError_t e = cudaLaunchKernelEx(&cfg, select_kernel, L, hdr);
   if (e != cudaSuccess) return e;
   if (L.in_place) {
@@ -456,6 +457,7 @@ cudaError_t launch_compact(const CompactLaunch &L, WsHeader *hdr, cudaStream_t s
     dim3 grid(2, L.M * L.H, L.n_traj);
     if (aligned) gather_in_place_kernel<16, 64><<<grid, 256, 0, stream>>>(L);
     else gather_in_place_kernel<2, 8><<<grid, 256, 0, stream>>>(L);
+    launch_count() += 2;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     positions_in_place_kernel<<<L.n_traj, 256, 0, stream>>>(L);
@@ -482,6 +484,7 @@ cudaError_t launch_compact(const CompactLaunch &L, WsHeader *hdr, cudaStream_t s
     dim3 grid((unsigned)((threads + 255) / 256), L.M * L.H, L.n_traj);
     gather_kernel<2><<<grid, 256, 0, stream>>>(L);
   }
+  ++launch_count();
   return cudaGetLastError();
 }
 

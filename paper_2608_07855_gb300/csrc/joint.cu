@@ -457,6 +457,7 @@ cudaError_t launch_joint_typed(const JointLaunch &L, WsHeader *hdr, cudaStream_t
   if (grid > ngroups) grid = ngroups;
   if (grid < 1) return cudaSuccess;
   void *args[] = {(void *)&L, (void *)&hdr};
+  ++launch_count();
   return cudaLaunchCooperativeKernel((const void *)joint_kernel<T, D>, dim3(grid), dim3(kThreads),
                                      args, smem, s);
 }
@@ -467,6 +468,7 @@ cudaError_t launch_joint_init(const JointLaunch &L, size_t rows, WsHeader *hdr, 
   const int64_t work = (int64_t)rows * L.batch.d / 4;
   const int64_t blocks = work < 256 ? 1 : work / 256 < 608 ? work / 256 : 608;
   joint_init_kernel<<<(unsigned)blocks, 256, 0, stream>>>(L, (int64_t)rows, hdr);
+  ++launch_count();
   return cudaGetLastError();
 }
 
@@ -498,6 +500,7 @@ extern "C" commitkv_status commitkv_test_barrier_timeout(void *workspace, size_t
   if (cudaMemsetAsync(&hdr->abort, 0, 3 * sizeof(int32_t), stream) != cudaSuccess) return COMMITKV_ERR_CUDA;
   unsigned expected = (unsigned)blocks + 1;
   void *args[] = {(void *)&hdr, (void *)&expected};
+  ++ckv::launch_count();
   cudaError_t e = cudaLaunchCooperativeKernel((const void *)ckv::barrier_timeout_kernel, dim3(blocks),
                                               dim3(32), args, 0, stream);
   if (e != cudaSuccess) {

@@ -683,6 +683,7 @@ cudaError_t launch_joint_tc(const JointLaunch &L, WsHeader *hdr, cudaStream_t st
   const int grid = ngroups < sm_count ? ngroups : sm_count;
   if (grid < 1) return cudaSuccess;
   void *args[] = {(void *)&L, (void *)&hdr};
+  ++launch_count();
   return cudaLaunchCooperativeKernel((const void *)joint_tc_kernel, dim3(grid), dim3(kThreads), args, smem,
                                      stream);
 }

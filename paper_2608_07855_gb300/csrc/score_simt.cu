@@ -532,6 +532,7 @@ cudaError_t launch_typed(const ScoreLaunch &L, float *partials, WsHeader *hdr, c
   if (rows > 0) combine_kernel<D><<<(rows * 32 + kThreads - 1) / kThreads, kThreads, 0, s>>>(L, partials);
   int nb = L.unit_off_b[L.batch.n_traj];
   if (nb > 0) pass_b_kernel<T, D><<<nb, kThreads, smem, s>>>(L, hdr);
+  launch_count() += 1 + (na > 0) + (rows > 0) + (nb > 0);
   return cudaGetLastError();
 }
 

@@ -2072,6 +2072,7 @@ cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t s, int sm_c
     nb = nb < nb_items ? nb : nb_items;
     if (nb < 1 && nb_items > 0) return cudaErrorInvalidConfiguration;
     prep_kernel<<<L.n_traj, 1024, 0, s>>>(L, hdr);
+    launch_count() += 2;
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemsetAsync(L.a_done, 0, (size_t)L.slice_off[L.n_traj] * kCounterStride * 4, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(L.merged, 0, (size_t)L.slice_off[L.n_traj] * kCounterStride * 4, s);
@@ -2096,10 +2097,13 @@ cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t s, int sm_c
     }
   }
   prep_kernel<<<L.n_traj, 1024, 0, s>>>(L, hdr);
+  launch_count() += 1 + (na_items > 0);
   if (na_items > 0) pass_a<<<na_items < sm_count ? na_items : sm_count, L.prune ? 512 : 384, smem_a(), s>>>(L, hdr);
   const int rows = L.from_stats ? 0 : L.row_off[L.n_traj];
   if (rows > 0) combine_tc<<<(rows * 32 + 255) / 256, 256, 0, s>>>(L);
+  launch_count() += rows > 0;
   if (L.prune) {
+    launch_count() += 6;
     const int units = L.unit_off[L.n_traj];
     bound_kernel<<<L.bound_off[L.n_traj], 256, 0, s>>>(L);
     seed_kernel<<<L.seed_off[L.n_traj], 512, 0, s>>>(L);
@@ -2110,6 +2114,7 @@ cudaError_t launch_score_tc(TcLaunch &L, WsHeader *hdr, cudaStream_t s, int sm_c
     return cudaGetLastError();
   }
   if (nb_items > 0) pass_b_tc<<<nb_items < sm_count ? nb_items : sm_count, 512, smem_b(), s>>>(L, hdr);
+  launch_count() += nb_items > 0;
   return cudaGetLastError();
 }
 

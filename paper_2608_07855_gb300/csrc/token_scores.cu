@@ -427,6 +427,7 @@ cudaError_t launch_tc(const Batch &b, const float *const *stats, float *const *s
     }
     const int n = L.item_off[nb];
     if (n > 0) token_scores_tc<<<n < sm_count ? n : sm_count, 320, smem_bytes(), s>>>(L, hdr);
+    launch_count() += n > 0;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -447,6 +448,7 @@ cudaError_t launch_simt(const Batch &b, const float *const *stats, float *const 
   }
   const int n = S.blk_off[b.n_traj];
   if (n <= 0) return cudaSuccess;
+  ++launch_count();
   if (b.dtype == COMMITKV_BF16) {
     if (b.d == 128) token_scores_simt<__nv_bfloat16, 128><<<n, kSimtThreads, 0, s>>>(S);
     else token_scores_simt<__nv_bfloat16, 64><<<n, kSimtThreads, 0, s>>>(S);

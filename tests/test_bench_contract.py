@@ -1,5 +1,5 @@
-"""Host arithmetic of bench.py (CPU): the roofline terms per step, the
-launch count per step, and the peak it divides by."""
+"""Host arithmetic of bench.py (CPU): the roofline terms per step and the
+peak it divides by."""
 import json
 import os
 import types
@@ -20,18 +20,6 @@ def test_algorithmic_terms_of_the_qwen3_8b_32k_step():
     tokens = 32768 + (32768 + 4096 + 32)  # pre-commit cache + post-commit cache (window included)
     assert bpt * tokens == 10_272_374_784
     assert cfg.g == 4
-
-
-def test_launches_per_step():
-    """Tensor-core path: prep, flash pass, combine, page pass (one scoring
-    call over both caches of up to 8 trajectories), two classify kernels,
-    the joint test, select and gather."""
-    for n, cfg in ((1, synth.CONFIGS["qwen3_8b_32k"]), (16, synth.CONFIGS["ragged16"])):
-        buf = types.SimpleNamespace(cfg=cfg, trajs=[None] * n)
-        groups = (2 * n + 15) // 16
-        assert bench.buf_launches(buf) == 4 * groups + 2 + 1 + 2
-    tiny = types.SimpleNamespace(cfg=synth.CONFIGS["tiny"], trajs=[None])
-    assert bench.buf_launches(tiny) == 3 + 2 + 1 + 2
 
 
 def test_peaks_are_the_measured_ones():
