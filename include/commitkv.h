@@ -176,6 +176,13 @@ const char *commitkv_status_string(commitkv_status status);
  *                m = max scaled score, l = sum exp(s - m), n = number of
  *                visible tokens (stored as float), 0, then o_p[0..d).
  *                commitkv_joint_test needs these for the post-commit pass.
+ * Which kernels run: bf16 caches take the tensor cores where every cache of the
+ * call with tokens and probe rows is 16-byte aligned (pointers and strides) and
+ * has distinct heads and layers; other calls take the CUDA cores.  With 64
+ * channels a cache whose statistics are asked for takes the CUDA cores in any
+ * case, as do commitkv_page_effects_from_stats, commitkv_joint_test and
+ * commitkv_token_scores of that width.  So R of such a cache may differ by a few
+ * 1e-6 between a call with stats_out and one without.
  * -------------------------------------------------------------------- */
 commitkv_status commitkv_page_effects(const commitkv_shape *shape, int32_t n_traj,
                                       const commitkv_traj *trajs, const uint8_t *layer_mask,

@@ -501,15 +501,22 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   const size_t stats_size = stats_bytes(shape, n_traj, trajs), scratch = workspace_bytes - kAlign - stats_size;
 
   int CL = chunk_len_for(shape, nl, n_traj, trajs, scratch), RB = simt_rows_per_block(), PG = simt_pages_per_block();
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return cuda_status(e);
   // small calls: fewer pages per block, down to one, until there is a block
-  // per SM (half as many blocks, this line, twice as many: 2K tokens of one
-  // layer and two heads 24, 24 and 30 us; two layers of four heads, 1.5K
-  // tokens, W = 8: 53, 41 and 27 us)
+  // per SM.  More blocks spread the pages, but each stages its own 64-token
+  // tiles, so the optimum depends on how pages and tiles meet; over nine fp32
+  // shapes half as many blocks, this line and twice as many took, both caches,
+  // us: 24, 24, 32 (2K tokens, one layer, two heads); 53, 40, 28 (1.5K, two
+  // layers, four heads, W = 8); 20, 16, 16; 78, 64, 102; 70, 70, 75; 73, 83, 79;
+  // 74, 74, 82; 618, 619, 619; 36, 31, 44
   for (; PG > 1; PG /= 2) {
     int64_t blocks = 0;
     for (int t = 0; t < n_traj; ++t)
       blocks += (int64_t)nl * shape->kv_heads * cdiv(L.batch.g * trajs[t].W, RB) * cdiv(trajs[t].P, PG);
-    if (blocks >= 152) break;
+    if (blocks >= sms) break;
   }
   L.pages_per_block = PG;
   int g = L.batch.g, d = shape->head_dim;
@@ -541,8 +548,7 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
   L.from_stats = from_stats ? 1 : 0;
   for (int t = 0; t < n_traj; ++t) {  // R itself is cleared by the first kernel
     if (trajs[t].P == 0 || !L.headR[t]) continue;
-    cudaError_t e =
-        cudaMemsetAsync(L.headR[t], 0, (size_t)shape->layers * shape->q_heads * trajs[t].P * 4, stream);
+    e = cudaMemsetAsync(L.headR[t], 0, (size_t)shape->layers * shape->q_heads * trajs[t].P * 4, stream);
     if (e != cudaSuccess) return cuda_status(e);
   }
   WsHeader *hdr = static_cast<WsHeader *>(workspace);
@@ -551,10 +557,6 @@ commitkv_status page_effects_impl(const commitkv_shape *shape, int32_t n_traj, c
     return cuda_status(launch_score_simt(L, partials, hdr, stream));
   // tensor-core path: trajectories in launches of up to tc::kMaxTc
   static thread_local tc::TcLaunch T;
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return cuda_status(e);
   const bool fused = !from_stats && env_fused() && d == 128;
   int CLt = tc_chunk_len(n_traj, trajs);
   if (fused) {

@@ -99,13 +99,22 @@ size_t prune_item_bytes(int S, int P, int slices, int nrt);
 void prune_layout(TcPrune &p, char *base, int S, int P, int slices, int nrt);
 // The page pass is pruned when the pages average at least kMinPageTokens
 // tokens (bounds the bookkeeping, which is per page and row: with 36 layers,
-// 8 KV heads and 16K + 2K tokens the call takes 6.0 ms against 15.5 ms with
-// the full pass for pages of 2 tokens, 1.53 against 2.28 ms for 32, 1.76
-// against 2.05 ms for 256), and when the launch has kMinPruneWork (unit,
-// token) pairs: below, the extra launches cost more than they save (1 layer
-// of 16K + 2K tokens 180 against 133 us, 36 layers of 1.5K tokens 432 against
-// 390 us; 4 layers of 16K + 2K 308 against 354 us, 36 layers of 4K 674
-// against 855 us).
+// 8 KV heads and 16K + 2K tokens the call takes 5.8 ms against 15.6 ms with
+// the full pass for pages of 2 tokens, 1.48 against 2.24 ms for 32, 1.76
+// against 1.99 ms for 256), and when the launch has kMinPruneWork (unit,
+// token) pairs: below, the extra launches cost more than they save.  Pruned
+// against full, us, 128 probe rows a unit: 2^18.1 pairs (1 layer of 16K + 2K
+// tokens) 176 and 126, 2^19.1 (2 layers) 214 and 210, 2^19.6 (36 layers of
+// 1.2K + 0.3K) 379 and 343, 2^20.1 (4 layers of 16K + 2K) 287 and 332, 2^20.4
+// (64 layers of 1.2K + 0.3K) 608 and 579, 2^21.3 (36 layers of 4K + 0.5K) 684
+// and 870.  32 of a unit's 128 rows: 2^18.1 201 and 149, 2^19.1 251 and 255,
+// 2^19.6 300 and 336, 2^20.1 336 and 392, 2^20.4 458 and 560, 2^21.3 648 and 1,000.
+// What is dropped depends on the data, which no rule here sees.  Where
+// nothing is (keys all alike) the sums, bounds and lists come on top of the
+// full pass: one cache of 18K tokens, 36 layers, in pages of 32 1,742 against
+// 1,585 us, of 16 2,439 against 2,133, of 100 and 250 1,602 against 1,490, of
+// 2 and 3 11.9 against 9.4 ms; 8 layers of 128K, 512 rows a KV head, 7.45
+// against 6.9 ms.  With random keys 1,298, 1,196, 1,604 us, 3.3 and 6.8 ms.
 constexpr int kMinPageTokens = 2;
 constexpr int64_t kMinPruneWork = 1 << 20;
 
