@@ -1294,8 +1294,9 @@ __device__ __forceinline__ void page_body(const TcLaunch &L, WsHeader *hdr, uint
   tc_fence_after();
   const uint32_t tm = sm.tmem;
   // read where it is compared: held in a register by every role it cost
-  // spills (the full page pass of 36 layers of 18K tokens in pages of 32: 884
-  // us, 872 so)
+  // spills (the full page pass of 36 layers of 18K tokens, in a register and
+  // so, us: pages of 32 tokens 884 and 872, of 100 and 250 784 and 777, of 16
+  // 1,408 and 1,417)
   const volatile int *count = &sm.ic.off[L.n_traj];
   auto n_items = [&]() { return LIST ? n_list : *count; };
 
