@@ -71,8 +71,8 @@ CASES = [
     (64, 8, 16, 4, 3000, [2800], "sharp"),  # one page of many tiles holding almost everything
     (64, 8, 16, 8, 2100, [2, 3], "normal"),
     (64, 8, 16, 8, 2100, [1, 2], "normal"),  # pages too short to prune: the full pass both times
-    (256, 16, 32, 32, 700, [16], "uniform"),  # units that keep everything, enough of them for items of two buckets
-    (128, 16, 32, 32, 1500, [16], "uniform"),  # the same with a third bucket alone
+    (128, 16, 32, 32, 1500, [16], "uniform"),  # units that keep everything, enough of them for items of two buckets
+    (128, 16, 32, 32, 2300, [16], "uniform"),  # the same with a third bucket alone
 ]
 
 
@@ -100,9 +100,12 @@ def _both(trajs, M, Hq, mask=None, prunes=True, most=1.0):
 @pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[6]}-{c[4]}-{c[5][0]}")
 def test_pruned_effects_equal_the_full_pass(case, d):
     M, H, Hq, W, S, sizes, kind = case
-    short = sizes == [1, 2]
-    t = _traj(M, H, Hq, d, S, W, sizes, kind, d + 1, 0 if short else 60)
+    short, whole = sizes == [1, 2], (sizes, kind) == ([16], "uniform")
+    t = _traj(M, H, Hq, d, S, W, sizes, kind, d + 1, 0 if short or whole else 60)
     assert (2 * t.page_start.numel() > S) == short
+    if whole:  # eight items of 128 slots a SM, from units that drop nothing
+        slots = int(((t.page_len + 15) // 16).sum()) * M * H * (-(-Hq // H * W // 128))
+        assert slots >= 8 * 128 * torch.cuda.get_device_properties(0).multi_processor_count
     # a fifth to three fifths is scored of the sharp caches with many pages, a hundredth of short pages
     most = 0.75 if kind == "sharp" and len(t.page_start) > 1 else 0.05 if sizes == [2, 3] else 1.0
     pruned, full = _both([t], M, Hq, prunes=not short, most=most)
