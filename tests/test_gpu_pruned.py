@@ -123,6 +123,14 @@ def test_pruned_effects_of_a_ragged_batch_with_a_layer_mask():
             assert np.array_equal(a, b)
 
 
+def test_pruned_effects_of_two_launches():
+    """18 caches take two launches, which use one region of tables in turn."""
+    trajs = [_traj(128, 8, 16, 128, 140 + 7 * i if i < 16 else 700 + i, 8, [16], "sharp", i, 4) for i in range(18)]
+    pruned, full = _both(trajs, 128, 16)
+    for a, b in zip(pruned, full):
+        assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("M,H,Hq,d,dtype,S,W,P,size", [(64, 8, 32, 128, "bfloat16", 2200, 8, 130, 112596992),
                                                        (16, 2, 8, 64, "bfloat16", 2200, 8, 130, 3064320),
                                                        (1, 2, 4, 64, "float32", 2300, 16, 140, 192000)],
